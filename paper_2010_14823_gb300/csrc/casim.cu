@@ -21,6 +21,7 @@
 
 #include "casim.h"
 #include "casim_device.cuh"
+#include "casim_step.cuh"
 #include "casim_batch.cuh"
 #include "casim_mlp.cuh"
 
@@ -218,21 +219,6 @@ static bool params_ok(const casim_params &p) {
   return true;
 }
 
-// a staged step kernel (in place, its whole-line-store form, source-term
-// mode) may use the dynamic shared memory of a column of the largest level count
-template <class M>
-static cudaError_t allow_step_smem() {
-  cudaError_t e = cudaFuncSetAttribute(k_step<M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)step_smem_bytes<M, false>(kMaxLev));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_step<M, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)step_smem_bytes<M, false>(kMaxLev));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_step<M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)step_smem_bytes<M, true>(kMaxLev));
-  return e;
-}
-
 extern "C" int casim_init(casim_ctx **out, const casim_params *params, int precision, int flags) {
   if (!out) return CASIM_ERR_ARG;
   *out = nullptr;
@@ -265,12 +251,12 @@ extern "C" int casim_init(casim_ctx **out, const casim_params *params, int preci
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->host_ro, cudaDevAttrHostRegisterReadOnlySupported, ctx->device);
   // the staged mixed steps' dynamic shared memory (prefetch stage and level
   // tables) exceeds the default 48 KB for long columns
-  if (e == cudaSuccess) e = allow_step_smem<PolicyMix>();
-  if (e == cudaSuccess) e = allow_step_smem<PolicyMixWarm>();
-  if (e == cudaSuccess) e = allow_step_smem<PolicyMixWarmAero>();
-  if (e == cudaSuccess) e = allow_step_smem<PolicyMixWarm3>();
-  if (e == cudaSuccess) e = allow_step_smem<PolicyMixAero>();
-  if (e == cudaSuccess) e = allow_step_smem<PolicyMix3>();
+  if (e == cudaSuccess) e = StepCold::allow_smem();
+  if (e == cudaSuccess) e = StepWarm::allow_smem();
+  if (e == cudaSuccess) e = StepWarmAero::allow_smem();
+  if (e == cudaSuccess) e = StepWarm3::allow_smem();
+  if (e == cudaSuccess) e = StepAero::allow_smem();
+  if (e == cudaSuccess) e = Step3::allow_smem();
   // and the batched step's (256-thread blocks: a 64 KB stage)
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_step_batch<PolicyMix, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -278,9 +264,6 @@ extern "C" int casim_init(casim_ctx **out, const casim_params *params, int preci
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_step_batch<PolicyMix, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)batch_smem_bytes<PolicyMix>(kBatchMaxBlock, kMaxLev));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_step<PolicyMix, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)step_smem_bytes<PolicyMix, false>(kMaxLev));
   ctx->stats = (flags & CASIM_STATS) != 0;
   if (e == cudaSuccess && ctx->stats) e = cudaMalloc(&ctx->d_stats, kStatsWords * sizeof(unsigned long long));
   if (e == cudaSuccess && ctx->stats) e = cudaMemset(ctx->d_stats, 0, kStatsWords * sizeof(unsigned long long));
@@ -322,10 +305,10 @@ static KArgs make_args(const casim_ctx *ctx, const casim_state *s, int ncols, in
   a.dt = dt;
   a.surr = nullptr;
   a.stats = ctx->stats ? ctx->d_stats : nullptr;
+  a.segs = 1;
   return a;
 }
 
-// tend null: the in-place step; else the source-term mode
 // fields and precipitation rows of a context's state
 static int ctx_nfields(const casim_ctx *ctx) {
   if (ctx->aero) return ctx->warm ? CASIM_NFIELDS_AEROSOL : CASIM_NFIELDS_AEROSOL_COLD;
@@ -334,44 +317,19 @@ static int ctx_nfields(const casim_ctx *ctx) {
 }
 static int ctx_nprecip(const casim_ctx *ctx) { return CASIM_NPRECIP + (ctx->aero ? 1 : 0); }
 
-// one configuration's kernels: the in-place step, or (tend) the source-term
-// mode; line: the state is mapped host memory (the mixed step's whole-line
-// stores)
-template <class PMix, class PF64>
-static void launch_pair(const casim_ctx *ctx, dim3 grid, cudaStream_t st, const KArgs &a, double *tend, bool line) {
-  const KParams &kp = ctx->kp;
-  if constexpr (std::is_same<PMix, PolicyMix>::value) {
-    // the statistics build (a CASIM_STATS context: standard configuration)
-    if (a.stats && !tend) {
-      if (ctx->precision == CASIM_MIXED)
-        k_step<PMix, false, true><<<grid, kBlock, step_smem_bytes<PMix, false>(a.nlev), st>>>(a, kp, nullptr);
-      else
-        k_step<PF64, false, true><<<grid, kBlock, step_smem_bytes<PF64, false>(a.nlev), st>>>(a, kp, nullptr);
-      return;
-    }
-  }
-  if (ctx->precision == CASIM_MIXED) {
-    if (tend) k_step<PMix, true><<<grid, kBlock, step_smem_bytes<PMix, true>(a.nlev), st>>>(a, kp, tend);
-    else if (line)
-      k_step<PMix, false, false, true><<<grid, kBlock, step_smem_bytes<PMix, false>(a.nlev), st>>>(a, kp, nullptr);
-    else k_step<PMix, false><<<grid, kBlock, step_smem_bytes<PMix, false>(a.nlev), st>>>(a, kp, nullptr);
-  } else {
-    if (tend) k_step<PF64, true><<<grid, kBlock, step_smem_bytes<PF64, true>(a.nlev), st>>>(a, kp, tend);
-    else k_step<PF64, false><<<grid, kBlock, step_smem_bytes<PF64, false>(a.nlev), st>>>(a, kp, nullptr);
-  }
-}
-
-static int launch_step(casim_ctx *ctx, const KArgs &a, int ncols, double *tend, void *stream, bool line = false) {
-  const dim3 grid((unsigned)((ncols + kBlock - 1) / kBlock));
-  cudaStream_t st = (cudaStream_t)stream;
-  if (ctx->aero && ctx->warm) launch_pair<PolicyMixWarmAero, PolicyF64WarmAero>(ctx, grid, st, a, tend, line);
-  else if (ctx->aero) launch_pair<PolicyMixAero, PolicyF64Aero>(ctx, grid, st, a, tend, line);
-  else if (ctx->tri && ctx->warm) launch_pair<PolicyMixWarm3, PolicyF64Warm3>(ctx, grid, st, a, tend, line);
-  else if (ctx->tri) launch_pair<PolicyMix3, PolicyF643>(ctx, grid, st, a, tend, line);
-  else if (ctx->warm) launch_pair<PolicyMixWarm, PolicyF64Warm>(ctx, grid, st, a, tend, line);
-  else launch_pair<PolicyMix, PolicyF64>(ctx, grid, st, a, tend, line);
+// the context's configuration; tend: the source-term mode; line: the state is
+// mapped host memory
+static int launch_step(casim_ctx *ctx, const KArgs &a, double *tend, void *stream, bool line = false) {
+  const StepLaunch l{ctx->precision == CASIM_MIXED, line, ctx->nsm, (cudaStream_t)stream, tend};
+  cudaError_t e;
+  if (ctx->aero && ctx->warm) e = StepWarmAero::launch(l, a, ctx->kp);
+  else if (ctx->aero) e = StepAero::launch(l, a, ctx->kp);
+  else if (ctx->tri && ctx->warm) e = StepWarm3::launch(l, a, ctx->kp);
+  else if (ctx->tri) e = Step3::launch(l, a, ctx->kp);
+  else if (ctx->warm) e = StepWarm::launch(l, a, ctx->kp);
+  else e = StepCold::launch(l, a, ctx->kp);
   ctx->launches++;
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(e);
   return CASIM_OK;
 }
 
@@ -388,7 +346,7 @@ extern "C" int casim_step_tendency(casim_ctx *ctx, const casim_state *s, int nco
       (tend < s->fld + span && s->fld < tend + tspan))   // must not overlap the state
     return CASIM_ERR_ARG;
   const KArgs a = make_args(ctx, s, ncols, nlev, dt);
-  return launch_step(ctx, a, ncols, tend, stream);
+  return launch_step(ctx, a, tend, stream);
 }
 
 // line: the state is mapped host memory
@@ -397,7 +355,7 @@ static int step_device(casim_ctx *ctx, const casim_state *s, int ncols, int nlev
   int rc = check_state(s, ncols, nlev, dt);
   if (rc != CASIM_OK || ncols == 0) return rc;
   const KArgs a = make_args(ctx, s, ncols, nlev, dt);
-  return launch_step(ctx, a, ncols, nullptr, stream, line);
+  return launch_step(ctx, a, nullptr, stream, line);
 }
 
 // a CASIM_STATS context counts the step and its points on the host
@@ -601,6 +559,23 @@ extern "C" int casim_step_host(casim_ctx *ctx, const casim_state *h, int ncols, 
   if (e != cudaSuccess) return cuda_fail(e, "casim_step_host");
   if (rc == CASIM_OK) count_step(ctx, ncols, nlev);
   return rc;
+}
+
+// Per-column FP64 budgets: water path and aerosol + droplet number path.
+static __global__ void __launch_bounds__(256) k_budget(const KArgs a, double *out) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= a.ncols) return;
+  double wsum = 0.0, nsum = 0.0;
+  const size_t fs = (size_t)a.nlev * (size_t)a.pitch;
+  for (int k = 0; k < a.nlev; ++k) {
+    const size_t o = (size_t)k * a.pitch + c;
+    const double m = a.fld[14 * fs + o] * a.dz[k];
+    wsum += m * (((((a.fld[1 * fs + o] + a.fld[2 * fs + o]) + a.fld[3 * fs + o]) + a.fld[4 * fs + o]) +
+                  a.fld[5 * fs + o]) + a.fld[6 * fs + o]);
+    nsum += m * (a.fld[7 * fs + o] + a.fld[12 * fs + o]);
+  }
+  out[c] = wsum;
+  out[(size_t)a.ncols + c] = nsum;
 }
 
 extern "C" int casim_budget(casim_ctx *ctx, const casim_state *s, int ncols, int nlev, double *out, void *stream) {
@@ -1709,10 +1684,9 @@ extern "C" int casim_step_surrogate(casim_ctx *ctx, casim_mlp *m, const casim_st
   }
   // 3. the step, taking the network's rates where given
   a.surr = m->surr;
-  const dim3 grid((unsigned)((ncols + kBlock - 1) / kBlock));
-  k_step<PolicyMix, false><<<grid, kBlock, step_smem_bytes<PolicyMix, false>(nlev), st>>>(a, ctx->kp, nullptr);
+  a.stats = nullptr;
   ctx->launches++;
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(StepCold::launch(StepLaunch{true, false, ctx->nsm, st, nullptr}, a, ctx->kp));
   if (served) *served = rows;
   return CASIM_OK;
 }

@@ -148,18 +148,11 @@ __global__ void __launch_bounds__(kNarrow ? kBatchNarrowBlock : kBatchMaxBlock,
     const DomDesc d = b.dom[item.dom];
     const int n = b.compact ? b.count[item.dom] : d.ncols;
     if (item.chunk * B < n) {
-      if (item.dom != prev_dom) {
-        for (int k = tid; k < d.nlev; k += B) level_tab(s_dz, s_dzdt, s_dtdz_f, s_dzdt_f, k, d.dz[k], b.dt);
-        __syncthreads();
-        prev_dom = item.dom;
-      }
-      bool fast = true;
-#pragma unroll
-      for (int x = 1; x < 5; ++x) fast &= ((P.vmax[x] * b.dt) / d.dzmin) / P.c_max <= 1.0;
       const int idx = item.chunk * B + tid;
+      KArgs a;
+      int c = 0;
       if (idx < n) {
-        const int c = b.compact && CASIM_INDEX_OK(idx < d.ncols, b.err) ? b.list[d.list_off + idx] : idx;
-        KArgs a;
+        c = b.compact && CASIM_INDEX_OK(idx < d.ncols, b.err) ? b.list[d.list_off + idx] : idx;
         a.fld = d.fld;
         a.pitch = d.pitch;
         a.dz = d.dz;
@@ -170,8 +163,20 @@ __global__ void __launch_bounds__(kNarrow ? kBatchNarrowBlock : kBatchMaxBlock,
         a.dt = b.dt;
         a.surr = b.surr ? b.surr + d.pt_off : nullptr;
         a.stats = nullptr;
-        eflag |= run_column<M, false, kStage>(a, P, lt, fast, c, nullptr, kStage ? stage + tid : nullptr, B);
+        a.segs = 1;
+        if (kStage) stage_level<M>(a, d.nlev - 1, c, stage + tid, B);   // in flight while the tables are made
       }
+      if (item.dom != prev_dom) {
+        for (int k = tid; k < d.nlev; k += B) level_tab(s_dz, s_dzdt, s_dtdz_f, s_dzdt_f, k, d.dz[k], b.dt);
+        __syncthreads();
+        prev_dom = item.dom;
+      }
+      bool fast = true;
+#pragma unroll
+      for (int x = 1; x < 5; ++x) fast &= one_substep(P.vmax[x], b.dt, d.dzmin, P.c_max);
+      if (idx < n)
+        eflag |= run_column<M, false, kStage, false, false, false>(a, P, lt, fast, c, Segment<false>(d.nlev), nullptr,
+                                                                   nullptr, kStage ? stage + tid : nullptr, B, nullptr);
     }
     // shared memory (item, dz) is reused by the next item; with one item per
     // block there is none, and the warps leave as they finish

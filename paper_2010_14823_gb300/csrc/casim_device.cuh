@@ -95,6 +95,7 @@ struct KArgs {
   double dt;
   const float4 *surr;   // [nlev][pitch] surrogate warm-rain rates (mixed form), or null
   unsigned long long *stats;   // per-step statistics (the statistics build of the step), or null
+  int segs;             // split step: level segments of a column per block (1, 2 or 4)
 };
 
 // Per-step statistics of one column: points the activity flag sent through
@@ -458,6 +459,23 @@ struct Shape3 {
   }
 };
 
+// Sums of products in the mixed limiter.  Whether one of the products goes
+// into the sum unrounded (a fused multiply-add) moves the sum by one FP32
+// rounding, and the compiler's own choice follows the uses a product has in
+// the kernel at hand: two kernels of one configuration could differ in the
+// last bit of a limited transfer.  So the choice is written out; `kFused` has
+// a bit per place, set as each configuration's kernels have always had it.
+template <bool kFused>
+__device__ __forceinline__ float add_product(float s, float a, float b) {   // s + a b
+  if constexpr (kFused) return fmaf(a, b, s);
+  else return __fadd_rn(s, __fmul_rn(a, b));
+}
+template <class M, bool kTend>
+__host__ __device__ constexpr unsigned limiter_fused() {
+  if (!M::kWarm) return M::kAero || M::kTri ? 15u : kTend ? 13u : 0u;
+  return kTend && (M::kAero || M::kTri) ? 9u : 0u;
+}
+
 template <class M>
 struct Phys {
   using R = typename M::R;
@@ -617,6 +635,7 @@ struct Phys {
 
   // a10: per-pool limiting factors f_X = min(1, X / (S_X dt)); each transfer
   // takes the smallest factor of the pools it draws from.
+  template <bool kTend = false>
   static __device__ __forceinline__ void limits(const ConstK<R> &K, const W<R> &w, double dt, const Rt<R> &r,
                                                 Gt<R> &g) {
     const R dtr = M::toR(dt);
@@ -635,8 +654,17 @@ struct Phys {
     const R S_qv = ((g.nucm + g.depp[0]) + g.depp[1]) + g.depp[2];
     const R S_qc = ((r.aut + r.acc) + r.rim[0]) + r.rim[1];
     const R S_qr = r.evr;
-    const R S_nc = (((r.aut * g.rc + r.acc * g.rc) + r.scc) + r.rim[0] * g.rc) + r.rim[1] * g.rc;
-    const R S_nr = r.scr + r.evr * g.rr;
+    R S_nc, S_nr;
+    if constexpr (!M::kMixed) {
+      S_nc = (((r.aut * g.rc + r.acc * g.rc) + r.scc) + r.rim[0] * g.rc) + r.rim[1] * g.rc;
+      S_nr = r.scr + r.evr * g.rr;
+    } else {
+      constexpr unsigned kFused = limiter_fused<M, kTend>();
+      S_nc = add_product<(kFused & 1u) != 0>(__fmul_rn(r.acc, g.rc), r.aut, g.rc) + r.scc;
+      S_nc = add_product<(kFused & 2u) != 0>(S_nc, r.rim[0], g.rc);
+      S_nc = add_product<(kFused & 4u) != 0>(S_nc, r.rim[1], g.rc);
+      S_nr = add_product<(kFused & 8u) != 0>(r.scr, r.evr, g.rr);
+    }
     auto fac = [&](R S, R X) -> R {
       if constexpr (!M::kMixed) {
         return S * dtr > X ? M::mx(X, (R)0) / (S * dtr) : (R)1;
@@ -1000,10 +1028,11 @@ struct MixT {
   // a2..a10 on an active point: FP32 throughout, except the initial vapour
   // difference of the adjustment, formed in FP64.  `surr`, if not null,
   // points at this point's surrogate warm-rain rates (NaN: use the scheme's).
+  template <bool kTend = false>
   static __device__ __forceinline__ void process(const ConstK<float> &K, const Pt &s, double dt, W<float> &w,
                                                  float es0, float qs0, MixInc &o, const float4 *surr = nullptr) {
     const float dnc_act = pre(K, s, w, es0, qs0, o);
-    post(K, w, dt, dnc_act, o, surr);
+    post<kTend>(K, w, dt, dnc_act, o, surr);
   }
 
   // a2 and a3; returns the cloud droplets activated
@@ -1109,6 +1138,7 @@ struct MixT {
   }
 
   // a4..a10 from the post-activation values
+  template <bool kTend>
   static __device__ __forceinline__ void post(const ConstK<float> &K, W<float> &w, double dt, float dnc_act,
                                               MixInc &o, const float4 *surr) {
     Rt<float> r;
@@ -1128,10 +1158,11 @@ struct MixT {
       }
     }
     Gt<float> g;
-    P::limits(K, w, dt, r, g);
+    P::template limits<kTend>(K, w, dt, r, g);
     const float dtr = d2f(dt);
-    o.cr = (g.aut * r.aut + g.acc * r.acc) * dtr;
-    o.cg = (g.rs * r.rim[0] + g.rg * r.rim[1]) * dtr;
+    // (rounded products: see add_product)
+    o.cr = __fmul_rn(add_product<false>(__fmul_rn(g.aut, r.aut), g.acc, r.acc), dtr);
+    o.cg = __fmul_rn(add_product<false>(__fmul_rn(g.rs, r.rim[0]), g.rg, r.rim[1]), dtr);
     o.rv = g.evr * r.evr * dtr;
     if constexpr (M::kTri) {
       o.r_aut = g.aut * r.aut * dtr;
@@ -1578,57 +1609,77 @@ template <class M>
 __host__ __device__ constexpr size_t stage_bytes(int block) {
   return 2 * (size_t)stage_nf<M>() * block * sizeof(double);
 }
-template <class M, bool kTend>
+// the split step's exchange slots, where the policy has no stage (one with a
+// stage uses the stage's, free by then): per thread one per sedimenting species
+__host__ __device__ constexpr size_t xch_bytes(int block) { return 4 * (size_t)block * sizeof(double); }
+template <class M, bool kTend, bool kSplit>
+__host__ __device__ constexpr size_t step_stage_bytes() {
+  return step_staged<M, kTend>() ? stage_bytes<M>(kBlock) : kSplit ? xch_bytes(kBlock) : 0;
+}
+template <class M, bool kTend, bool kSplit>
 __host__ __device__ constexpr size_t step_smem_bytes(int nlev) {
-  return (step_staged<M, kTend>() ? stage_bytes<M>(kBlock) : 0) + (size_t)nlev * 24 + (kBlock / 32) * 8 + 16;
+  return step_stage_bytes<M, kTend, kSplit>() + (size_t)nlev * 24 + (kBlock / 32) * 8;
 }
 
 struct StepSmem {
-  double *stage;   // [2][16][kBlock] or null
+  double *stage;   // [2][fields][kBlock], or the exchange slots [4][kBlock] of a policy without a stage
   LevelTab lt;
   double *red;
-  int *fast;
 };
 
-template <class M, bool kTend>
+template <class M, bool kTend, bool kSplit>
 __device__ __forceinline__ StepSmem step_smem(unsigned char *base, int nlev) {
   StepSmem m;
   unsigned char *p = base;
-  m.stage = nullptr;
-  if constexpr (step_staged<M, kTend>()) {
-    m.stage = reinterpret_cast<double *>(p);
-    p += stage_bytes<M>(kBlock);
-  }
+  m.stage = reinterpret_cast<double *>(p);
+  p += step_stage_bytes<M, kTend, kSplit>();
   double *dz = reinterpret_cast<double *>(p), *dzdt = dz + nlev;
   float *dtdz_f = reinterpret_cast<float *>(dzdt + nlev), *dzdt_f = dtdz_f + nlev;
   m.lt = LevelTab{dz, dzdt, dtdz_f, dzdt_f};
   m.red = reinterpret_cast<double *>(dzdt_f + nlev);   // 24 nlev bytes in: 8-byte aligned
-  m.fast = reinterpret_cast<int *>(m.red + kBlock / 32);
   return m;
 }
 
+// vmax dt / dzmin / c_max <= 1: a species' capped speed keeps within one level
+// per step.  The two FP64 divisions only decide within 0.1 % of the limit.
+__device__ __forceinline__ bool one_substep(double vmax, double dt, double dzmin, double c_max) {
+  const double v = vmax * dt, lim = dzmin * c_max;
+  if (v < 0.999 * lim) return true;
+  if (v > 1.001 * lim) return false;
+  return v / dzmin / c_max <= 1.0;
+}
+
 // Block prologue: the level tables into shared memory, and whether every
-// species' capped speed keeps within one level per step.
-__device__ __forceinline__ bool prologue(const KArgs &a, const KParams &P, const StepSmem &sm) {
+// species' capped speed keeps within one level per step.  kSplit: the tables
+// of the block's levels k0..k1 only, all of them in the multi-substep path.
+template <bool kSplit>
+__device__ __forceinline__ bool prologue(const KArgs &a, const KParams &P, const StepSmem &sm, int k0, int k1) {
   double dzmin = 1e300;
-  for (int k = threadIdx.x; k < a.nlev; k += blockDim.x) {
-    const double v = a.dz[k];
+  auto table = [&](int k, double v) {
     level_tab(const_cast<double *>(sm.lt.dz), const_cast<double *>(sm.lt.dzdt), const_cast<float *>(sm.lt.dtdz_f),
               const_cast<float *>(sm.lt.dzdt_f), k, v, a.dt);
+  };
+  for (int k = threadIdx.x; k < a.nlev; k += blockDim.x) {
+    const double v = a.dz[k];
+    if (!kSplit || (k >= k0 && k <= k1)) table(k, v);
     dzmin = fmin(dzmin, v);
   }
   for (int o = 16; o > 0; o >>= 1) dzmin = fmin(dzmin, __shfl_xor_sync(0xffffffffu, dzmin, o));
   if ((threadIdx.x & 31) == 0) sm.red[threadIdx.x >> 5] = dzmin;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  bool fast = true;
+  if ((threadIdx.x & 31) < 4) {   // one species per lane
     double m = sm.red[0];
     for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = fmin(m, sm.red[i]);
-    int fast = 1;
-    for (int x = 1; x < 5; ++x) fast &= ((P.vmax[x] * a.dt) / m) / P.c_max <= 1.0;
-    *sm.fast = fast;
+    fast = one_substep(P.vmax[1 + (threadIdx.x & 31)], a.dt, m, P.c_max);
   }
-  __syncthreads();
-  return *sm.fast != 0;
+  fast = __all_sync(0xffffffffu, fast);
+  if (kSplit && !fast) {
+    for (int k = threadIdx.x; k < a.nlev; k += blockDim.x)
+      if (k < k0 || k > k1) table(k, a.dz[k]);
+    __syncthreads();
+  }
+  return fast;
 }
 
 // 8-byte asynchronous copy global -> shared (this thread's own slot)
@@ -1639,6 +1690,44 @@ __device__ __forceinline__ void cp_async8(double *dst, const double *src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Split step: several threads share a column, each a segment of its levels.
+// Their warps are the warps of a block, of a cluster of blocks, or both; this
+// barrier joins them: arrive orders a thread's earlier accesses before it,
+// wait the later ones after it (exited threads count as arrived).
+__device__ __forceinline__ void split_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void split_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// The levels one thread handles: ktop down to kbot; kfirst is the level it
+// starts from, the one above ktop where it has to work out the flux into its
+// segment.  Segment 0 is at the top.
+template <bool kSplit>
+struct Segment {
+  int nlev;
+  __device__ explicit Segment(int n) : nlev(n) {}
+  __device__ __forceinline__ int ktop() const { return nlev - 1; }
+  __device__ __forceinline__ int kbot() const { return 0; }
+  __device__ __forceinline__ int kfirst() const { return nlev - 1; }
+};
+template <>
+struct Segment<true> {
+  int seg, nseg, segs, top, bot;
+  __device__ Segment(int nlev, int seg_, int nseg_, int segs_)
+      : seg(seg_), nseg(nseg_), segs(segs_), top(nlev - 1 - seg_ * nlev / nseg_), bot(nlev - (seg_ + 1) * nlev / nseg_) {}
+  __device__ __forceinline__ int ktop() const { return top; }
+  __device__ __forceinline__ int kbot() const { return bot; }
+  __device__ __forceinline__ int kfirst() const { return top + (seg > 0); }
+  // the exchange slot of segment j of this thread's column (`mine`: this
+  // thread's own): segs segments per block, the blocks of a cluster in order
+  __device__ __forceinline__ double slot(const double *mine, int j) const {
+    const double *p = mine + (j % segs - seg % segs) * ((int)blockDim.x / segs);
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(j / segs));
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+    return v;
+  }
+};
 
 // largest Courant number of each species so far, with the point's processed
 // values (multi-substep path): the substep count follows from its maximum
@@ -1665,6 +1754,17 @@ __device__ __forceinline__ void courant(const KArgs &a, const ConstK<typename M:
     }
     cmax[x] = M::mx(cmax[x], M::div(vq * M::toR(a.dt), M::toR(sdz[k])));
   }
+}
+
+// start copying level k of column c into this thread's stage slots
+template <class M>
+__device__ __forceinline__ void stage_level(const KArgs &a, int k, int c, double *slots, int ss) {
+  if (!CASIM_INDEX_OK(k >= 0 && k < a.nlev && c >= 0 && c < a.ncols && c < a.pitch, a.err)) return;
+  const size_t fs = (size_t)a.nlev * (size_t)a.pitch;
+  const double *src = a.fld + (size_t)k * a.pitch + c;
+#pragma unroll
+  for (int i = 0; i < stage_nf<M>(); ++i) cp_async8(slots + i * ss, src + stage_field<M>(i) * fs);
+  cp_async_commit();
 }
 
 // Multi-substep sedimentation of species x of one column after the processes
@@ -1820,19 +1920,30 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
 // those of the in-place step.
 // fast: the single-substep path, an instantiation of its own, so that neither
 // path's loop carries the other's instructions
-template <class M, bool fast, bool kTend, bool kStage, bool kStats, bool kLine>
+// sg: the levels this thread handles.  A thread of a lower segment first works
+// out the flux into its segment from the level above it, without storing that
+// level: the flux out of a level depends on that level's own point alone, so
+// it comes out bit for bit as in the thread that owns the level.  The barrier
+// keeps an owner from storing its lowest level before the thread below has
+// read it.  xch: this thread's exchange slots (stride ss), one per
+// sedimenting species.
+template <class M, bool fast, bool kTend, bool kStage, bool kStats, bool kLine, bool kSplit>
 __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &P, const LevelTab &lt, int c,
-                                                 double *tend, double *stg, int ss, ColStats *cs) {
+                                                 const Segment<kSplit> &sg, double *xch, double *tend, double *stg,
+                                                 int ss, ColStats *cs) {
   static_assert(!kLine || (kStage && !kTend && !kStats), "whole-line stores re-read the stage");
   const double *sdz = lt.dz, *sdzdt = lt.dzdt;
   constexpr int kNf = stage_nf<M>();
+  constexpr bool kShare = kSplit && fast && !kTend;   // the barrier above
+  const int kfirst = fast ? sg.kfirst() : sg.ktop();
   if constexpr (kStage) {
     if (!CASIM_INDEX_OK(c >= 0 && c < a.ncols && c < a.pitch, a.err)) return 0u;
-    const size_t fs = (size_t)a.nlev * (size_t)a.pitch;
-    const double *src = a.fld + (size_t)(a.nlev - 1) * a.pitch + c;
-#pragma unroll
-    for (int i = 0; i < kNf; ++i) cp_async8(stg + i * ss, src + stage_field<M>(i) * fs);
-    cp_async_commit();
+    if constexpr (kSplit && !fast) {
+      // no flux is carried here: the first level is ktop, not the one the
+      // caller staged
+      cp_async_wait<0>();
+      stage_level<M>(a, kfirst, c, stg, ss);
+    }
   }
   using R = typename M::R;
   using Ph = Phys<M>;
@@ -1851,19 +1962,14 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
   unsigned lvmask[kStats ? (kMaxLev + 31) / 32 : 1];
   if constexpr (kStats)
     for (int i = 0; i < (a.nlev + 31) / 32; ++i) lvmask[i] = 0u;
-  for (int k = a.nlev - 1; k >= 0; --k) {
+  for (int k = kfirst; k >= sg.kbot(); --k) {
     Pt s;
     const double *cur = nullptr;   // this level's slots of the stage (kStage)
     if constexpr (kStage) {
-      const int b = (a.nlev - 1 - k) & 1;
+      const int b = (kfirst - k) & 1;
       cur = stg + b * kNf * ss;
-      if (k > 0) {
-        double *nxt = stg + (b ^ 1) * kNf * ss;
-        const size_t fs = (size_t)a.nlev * (size_t)a.pitch;
-        const double *src = a.fld + (size_t)(k - 1) * a.pitch + c;
-#pragma unroll
-        for (int i = 0; i < kNf; ++i) cp_async8(nxt + i * ss, src + stage_field<M>(i) * fs);
-        cp_async_commit();
+      if (k > sg.kbot()) {
+        stage_level<M>(a, k - 1, c, stg + (b ^ 1) * kNf * ss, ss);
         cp_async_wait<1>();   // this level's copies (the older group) have landed
       } else {
         cp_async_wait<0>();
@@ -1881,6 +1987,9 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
       }
     } else {
       load_pt<M::kWarm, M::kAero, M::kTri>(a, k, c, s);
+    }
+    if constexpr (kShare) {
+      if (k == kfirst) split_arrive();   // the level above the segment has been read
     }
     bool touched;
     if constexpr (!M::kMixed) {
@@ -1956,7 +2065,7 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
       float dn[4] = {0.f, 0.f, 0.f, 0.f};   // number increments of r, i, s, g
       float qpost[4], npost[4];
       if (act) {
-        MixT<M>::process(K, s, a.dt, w, es0, qs0, o, a.surr ? a.surr + (size_t)k * a.pitch + c : nullptr);
+        MixT<M>::template process<kTend>(K, s, a.dt, w, es0, qs0, o, a.surr ? a.surr + (size_t)k * a.pitch + c : nullptr);
         if constexpr (kStage && !M::kWarm && !M::kAero && !M::kTri) {
           // the FP64 values the increments are added to, read again from this
           // level's stage slots (they stay there until the level after next is
@@ -2053,6 +2162,12 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
       eflag |= w.hmax >= kF32RangeHi;
     }
     if constexpr (!fast) courant<M>(a, K, sdz, k, s, Fq);   // the flux registers hold the Courant numbers
+    if constexpr (kSplit && fast) {
+      if (k > sg.ktop()) continue;   // the level above the segment: its flux only
+      if constexpr (kShare) {
+        if (k == sg.ktop()) split_wait();
+      }
+    }
     if constexpr (kTend) {
       eflag |= store_tend<M>(a, tend, k, c, s, fast, per_dt, kStage ? cur : nullptr, ss);
     } else if constexpr (kLine) {
@@ -2105,6 +2220,7 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
     }
   }
   if constexpr (fast) {
+    if (kSplit && sg.kbot() > 0) return eflag;   // the surface is another segment's
 #pragma unroll
     for (int x = 0; x < kSed; ++x) prec[x] = M::toD(Fq[x]) * a.dt;
     if constexpr (M::kAero) {
@@ -2113,8 +2229,23 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
       for (int x = 0; x < na3<M>(); ++x) prec[4] += M::toD(Fa[x]) * a.dt;
     }
   } else {
-    for (int x = 0; x < kSed; ++x) {
-      int ns = (int)ceil((double)M::div(x == 0 ? Fq[0] : x == 1 ? Fq[1] : x == 2 ? Fq[2] : Fq[3], M::toR(P.c_max)));
+    // split step: the segments' Courant numbers meet, and the species are
+    // dealt to the column's threads (with aerosol mass one thread takes them
+    // all: their surface fluxes of aerosol add up in order)
+    int x0 = 0, dx = 1;
+    if constexpr (kSplit) {
+#pragma unroll
+      for (int x = 0; x < kSed; ++x) xch[x * ss] = M::toD(Fq[x]);
+      split_arrive();
+      split_wait();
+      x0 = M::kAero && sg.seg > 0 ? kSed : sg.seg;
+      dx = M::kAero ? 1 : sg.nseg;
+    }
+    for (int x = x0; x < kSed; x += dx) {
+      R cmax = x == 0 ? Fq[0] : x == 1 ? Fq[1] : x == 2 ? Fq[2] : Fq[3];
+      if constexpr (kSplit)
+        for (int j = 0; j < sg.nseg; ++j) cmax = M::mx(cmax, M::toR(sg.slot(xch + x * ss, j)));
+      int ns = (int)ceil((double)M::div(cmax, M::toR(P.c_max)));
       if (ns < 1) ns = 1;
       if (ns > 64) { ns = 64; eflag |= 2u; }
       if constexpr (kStats) cs->nsub[x] = ns;
@@ -2124,10 +2255,14 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
       for (int i = 0; i < kSed; ++i)
         if (x == i) prec[i] = pr;
     }
+    if constexpr (kSplit) {   // the slots have been read and the sweeps' results stored
+      split_arrive();
+      split_wait();
+    }
     if constexpr (kTend) {
       // tendency mode: the new state in tend becomes (x_new - x_old) / dt
       const size_t fs = (size_t)a.nlev * (size_t)a.pitch;
-      for (int k = 0; k < a.nlev; ++k) {
+      for (int k = sg.kbot(); k <= sg.ktop(); ++k) {
         const size_t o = (size_t)k * a.pitch + c;
 #pragma unroll
         for (int f = 0; f < 13; ++f) {
@@ -2157,12 +2292,13 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
   return eflag;
 }
 
-template <class M, bool kTend = false, bool kStage = false, bool kStats = false, bool kLine = false>
+// (kStage: the caller has staged level sg.kfirst() with stage_level)
+template <class M, bool kTend, bool kStage, bool kStats, bool kLine, bool kSplit>
 __device__ __forceinline__ unsigned run_column(const KArgs &a, const KParams &P, const LevelTab &lt, bool fast, int c,
-                                               double *tend = nullptr, double *stg = nullptr, int ss = kBlock,
-                                               ColStats *cs = nullptr) {
-  return fast ? sweep_column<M, true, kTend, kStage, kStats, kLine>(a, P, lt, c, tend, stg, ss, cs)
-              : sweep_column<M, false, kTend, kStage, kStats, kLine>(a, P, lt, c, tend, stg, ss, cs);
+                                               const Segment<kSplit> &sg, double *xch, double *tend, double *stg,
+                                               int ss, ColStats *cs) {
+  return fast ? sweep_column<M, true, kTend, kStage, kStats, kLine, kSplit>(a, P, lt, c, sg, xch, tend, stg, ss, cs)
+              : sweep_column<M, false, kTend, kStage, kStats, kLine, kSplit>(a, P, lt, c, sg, xch, tend, stg, ss, cs);
 }
 
 // one column's statistics into the buffer: warp sums, one atomic per warp
@@ -2187,40 +2323,44 @@ __device__ __forceinline__ void stats_add(unsigned long long *st, const ColStats
 }
 
 // kTend: tendency mode (tend receives the source terms, a.fld unchanged).
-// Dynamic shared memory: step_smem_bytes<M, kTend>(a.nlev).  kStats: the
+// Dynamic shared memory: step_smem_bytes<M, kTend, kSplit>(a.nlev).  kStats: the
 // statistics instantiation (standard configuration; a.stats set).  kLine:
-// whole-line stores for a state in mapped host memory (staged policies)
-template <class M, bool kTend, bool kStats = false, bool kLine = false>
+// whole-line stores for a state in mapped host memory (staged policies).
+//
+// kSplit: the levels of a column are shared by gridDim.y a.segs threads (the
+// rows of a cluster of gridDim.y blocks, a.segs of them in a block), for
+// domains whose columns alone leave the chip idle: a warp's level is a chain
+// of some 4 700 cycles, and one warp per scheduler took 50 of them one after
+// another.  Measured (mixed): 256 columns x 50 levels 114 -> 16 us, 20 000 x 60
+// 172 -> 90 us (step_segments has the line between the two).
+template <class M, bool kTend, bool kStats = false, bool kLine = false, bool kSplit = false>
 __global__ void __launch_bounds__(kBlock, M::kMinBlocks) k_step(const KArgs a, const KParams P, double *tend) {
   extern __shared__ __align__(16) unsigned char step_dyn[];
-  const StepSmem sm = step_smem<M, kTend>(step_dyn, a.nlev);
-  const bool fast = prologue(a, P, sm);
-  const int c = blockIdx.x * kBlock + threadIdx.x;
-  if (c >= a.ncols) return;
   constexpr bool kStage = step_staged<M, kTend>();
+  const StepSmem sm = step_smem<M, kTend, kSplit>(step_dyn, a.nlev);
   ColStats cs{0, 0, {1, 1, 1, 1}};
-  const unsigned eflag = run_column<M, kTend, kStage, kStats, kLine>(a, P, sm.lt, fast, c, tend,
-                                                                     kStage ? sm.stage + threadIdx.x : nullptr,
-                                                                     kBlock, &cs);
+  double *mine = sm.stage + threadIdx.x;
+  unsigned eflag;
+  if constexpr (kSplit) {
+    const int cols = kBlock / a.segs, nseg = gridDim.y * a.segs;
+    const int c = blockIdx.x * cols + (int)(threadIdx.x & (cols - 1));
+    const Segment<true> sg(a.nlev, blockIdx.y * a.segs + threadIdx.x / cols, nseg, a.segs);
+    const Segment<true> s0(a.nlev, blockIdx.y * a.segs, nseg, a.segs), s1(a.nlev, (blockIdx.y + 1) * a.segs - 1, nseg, a.segs);
+    if (kStage && c < a.ncols) stage_level<M>(a, sg.kfirst(), c, mine, kBlock);
+    const bool fast = prologue<true>(a, P, sm, s1.kbot(), s0.kfirst());
+    if (c >= a.ncols) return;
+    eflag = run_column<M, kTend, kStage, kStats, kLine, true>(a, P, sm.lt, fast, c, sg, mine, tend,
+                                                              kStage ? mine : nullptr, kBlock, &cs);
+  } else {
+    const int c = blockIdx.x * kBlock + threadIdx.x;
+    if (kStage && c < a.ncols) stage_level<M>(a, a.nlev - 1, c, mine, kBlock);
+    const bool fast = prologue<false>(a, P, sm, 0, 0);
+    if (c >= a.ncols) return;
+    eflag = run_column<M, kTend, kStage, kStats, kLine, false>(a, P, sm.lt, fast, c, Segment<false>(a.nlev), nullptr, tend,
+                                                               kStage ? mine : nullptr, kBlock, &cs);
+  }
   if constexpr (kStats) stats_add(a.stats, cs);
   if (eflag) atomicOr(a.err, eflag);
-}
-
-// Per-column FP64 budgets: water path and aerosol + droplet number path.
-__global__ void __launch_bounds__(256) k_budget(const KArgs a, double *out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= a.ncols) return;
-  double wsum = 0.0, nsum = 0.0;
-  const size_t fs = (size_t)a.nlev * (size_t)a.pitch;
-  for (int k = 0; k < a.nlev; ++k) {
-    const size_t o = (size_t)k * a.pitch + c;
-    const double m = a.fld[14 * fs + o] * a.dz[k];
-    wsum += m * (((((a.fld[1 * fs + o] + a.fld[2 * fs + o]) + a.fld[3 * fs + o]) + a.fld[4 * fs + o]) +
-                  a.fld[5 * fs + o]) + a.fld[6 * fs + o]);
-    nsum += m * (a.fld[7 * fs + o] + a.fld[12 * fs + o]);
-  }
-  out[c] = wsum;
-  out[(size_t)a.ncols + c] = nsum;
 }
 
 }  // namespace casim_dev

@@ -563,6 +563,7 @@ __global__ void __launch_bounds__(256) k_mlp_features_batch(const DomDesc *dom, 
     a.dt = dt;
     a.surr = nullptr;
     a.stats = nullptr;
+    a.segs = 1;
     feature_point(a, P, fa, g - d.pt_off, g, warm, f, y, mk);
   }
   feature_append(fa, warm, g, f, y, mk);
