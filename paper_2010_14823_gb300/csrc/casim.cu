@@ -1127,7 +1127,10 @@ struct casim_mlp {
   MlpBf16 wb{};
   __nv_bfloat16 *wbuf = nullptr;
   unsigned char *img = nullptr;   // weight images for the tcgen05 kernel
-  float *wsplit = nullptr;        // split-K partial weight gradients [kSplitMax][256][256]
+  float *wsplit = nullptr;        // split-K partial weight gradients (MlpGradWs)
+  float *bpart = nullptr;         // partial bias gradients [kColsumChunks][kColsumLen]
+  float *hist = nullptr;          // losses of a fit's steps
+  int cap_hist = 0;
   unsigned *d_err = nullptr;
   int engine = 1;                 // 1: tcgen05 inference, 0: mma.sync
   float *norm = nullptr;   // [12 mean][12 sd][4 mean][4 sd]
@@ -1190,6 +1193,8 @@ static int mlp_batch_ws(casim_mlp *m, int n) {
   if (e == cudaSuccess) e = dalloc(&m->Xn, (size_t)n * kNin);
   if (e == cudaSuccess) e = dalloc(&m->Tn, (size_t)n * kNout);
   if (e == cudaSuccess) e = dalloc(&m->Mb, (size_t)n * kNout);
+  // (columns 4.. of the output layer's BF16 gradient stay zero)
+  if (e == cudaSuccess) e = cudaMemset(m->dzb4, 0, (size_t)n * kNoutPad * sizeof(__nv_bfloat16));
   if (e != cudaSuccess) {
     mlp_free_batch(m);
     return e == cudaErrorMemoryAllocation ? CASIM_ERR_OOM : cuda_fail(e, "cudaMalloc");
@@ -1198,14 +1203,26 @@ static int mlp_batch_ws(casim_mlp *m, int n) {
   return CASIM_OK;
 }
 
-// the tcgen05 GEMM takes operands that are K-major or MN-major with
-// 16-byte aligned rows (strides in multiples of 8 elements)
-static bool tc_operands_ok(long long sr, long long sk) {
-  return (sk == 1 && sr % 8 == 0) || (sr == 1 && sk % 8 == 0);
+// Launch with programmatic stream serialisation: the kernel's prologue runs
+// while the one before it on the stream drains (it calls pdl_wait before it
+// touches memory).
+template <class... P, class... A>
+static void launch_pdl(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
-// one training GEMM: on the tensor-core engine (engine 1) the tcgen05 kernel,
-// else (or for operands it does not take) the mma.sync kernel
+// one training GEMM: on the tensor-core engine (engine 1) the tcgen05 kernel
+// (K-major operands with 16-byte aligned rows), else the mma.sync kernel
 template <class Epi>
 static void launch_gemm(const casim_mlp *m, const GemmArgs &g, const Epi &epi, int nsplit, cudaStream_t st);
 
@@ -1216,77 +1233,83 @@ static void gemm(const casim_mlp *m, const __nv_bfloat16 *A, long long sam, long
   launch_gemm(m, g, epi, 1, st);
 }
 
-// weight gradient out[m][n] (ld N) = sum_k A(m, k) B(n, k) over a long K (the
-// batch): K split into chunks (kSplitK rows on the mma.sync engine; on the
-// tensor-core engine 256, enough chunks to give every SM a tile), partial
-// tiles summed in order
-constexpr int kSplitK = 512, kSplitKTc = 256, kSplitMax = 64;
-static void gemm_wgrad(casim_mlp *m, const __nv_bfloat16 *A, long long sam, long long sak, const __nv_bfloat16 *B,
-                       long long sbn, long long sbk, int M, int N, int K, float *out, cudaStream_t st) {
-  const int split = m->engine == 1 ? kSplitKTc : kSplitK;
-  const int kchunk = std::max(split, (K + kSplitMax - 1) / kSplitMax + kGBK - 1) / kGBK * kGBK;
-  const int nsplit = (K + kchunk - 1) / kchunk;
-  GemmArgs g{A, sam, sak, B, sbn, sbk, M, N, K, kchunk};
-  const long long len = (long long)M * N;
-  launch_gemm(m, g, EpiPartial{m->wsplit, N, len}, nsplit, st);
-  k_splitk_sum<<<(unsigned)((len + 255) / 256), 256, 0, st>>>(m->wsplit, nsplit, len, out);
-}
-
 template <class Epi>
 static void launch_gemm(const casim_mlp *m, const GemmArgs &g, const Epi &epi, int nsplit, cudaStream_t st) {
-  if (m->engine == 1 && tc_operands_ok(g.sam, g.sak) && tc_operands_ok(g.sbn, g.sbk)) {
-    const dim3 grid((g.N + kTcBN - 1) / kTcBN, (g.M + kTcBM - 1) / kTcBM, nsplit);
-    k_gemm_tc<Epi><<<grid, 128, kTcSmem, st>>>(g, epi, m->d_err);
-  } else {
+  if constexpr (!std::is_same<Epi, EpiPartial>::value) {
+    if (m->engine == 1 && g.sak == 1 && g.sbk == 1 && g.sam % 8 == 0 && g.sbn % 8 == 0) {
+      const dim3 grid((g.N + kTcBN - 1) / kTcBN, (g.M + kTcBM - 1) / kTcBM);
+      launch_pdl(k_gemm_tc<Epi>, grid, kTcThreads, kTcSmem, st, g, epi, m->d_err);
+      return;
+    }
+  }
+  if constexpr (!std::is_same<Epi, EpiOutLoss>::value) {   // (engine 1 only)
     const dim3 grid((g.N + kGBN - 1) / kGBN, (g.M + kGBM - 1) / kGBM, nsplit);
     k_gemm<Epi><<<grid, 128, 0, st>>>(g, epi);
   }
 }
 
-// forward pass of n rows whose BF16 inputs are in m->h0; keep_act stores the
+// hidden layers of n rows whose BF16 inputs are in m->h0; keep_act stores the
 // FP32 activations the backward pass needs
-static void mlp_forward(casim_mlp *m, int n, bool keep_act, cudaStream_t st) {
+static void mlp_hidden(casim_mlp *m, int n, bool keep_act, cudaStream_t st) {
   gemm(m, m->h0, kNinPad, 1, m->wb.w1t, kNinPad, 1, n, kNh, kNinPad,
        EpiHidden{m->theta + kOffB1, keep_act ? m->a1 : nullptr, m->h1, kNh}, st);
   gemm(m, m->h1, kNh, 1, m->wb.w2t, kNh, 1, n, kNh, kNh, EpiHidden{m->theta + kOffB2, keep_act ? m->a2 : nullptr, m->h2, kNh}, st);
   gemm(m, m->h2, kNh, 1, m->wb.w3t, kNh, 1, n, kNh, kNh, EpiHidden{m->theta + kOffB3, keep_act ? m->a3 : nullptr, m->h3, kNh}, st);
+}
+
+// forward pass: outputs in m->y
+static void mlp_forward(casim_mlp *m, int n, cudaStream_t st) {
+  mlp_hidden(m, n, false, st);
   gemm(m, m->h3, kNh, 1, m->wb.w4t, kNh, 1, n, kNout, kNh, EpiOut{m->theta + kOffB4, m->y, kNout}, st);
 }
 
-// loss and gradient of n rows (inputs in h0, targets Tn, masks Mb)
-static void mlp_backward(casim_mlp *m, int n, cudaStream_t st) {
-  cudaMemsetAsync(m->cnt, 0, sizeof(float), st);
-  cudaMemsetAsync(m->loss, 0, sizeof(double), st);
-  k_sum<<<64, 256, 0, st>>>(m->Mb, (long long)n * kNout, m->cnt);
-  const long long tot = (long long)n * kNoutPad;
-  k_mlp_loss<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(m->y, m->Tn, m->Mb, n, m->cnt, m->loss, m->dz4, m->dzb4);
-  const dim3 cs(32, kColsumY);
-  // bias gradients: column sums over row chunks (into wsplit's tail), then in order
-  float *cpart = m->wsplit + (size_t)(kSplitMax - 1) * kNh * kNh;
-  auto colsum = [&](const float *dz, int cols, float *g) {
-    k_colsum<<<dim3((cols + 31) / 32, kColsumChunks), cs, 0, st>>>(dz, n, cols, cols, cpart);
-    k_colsum_fin<<<1, 256, 0, st>>>(cpart, kColsumChunks, cols, g);
-  };
-  // layer 4
-  gemm_wgrad(m, m->h3, 1, kNh, m->dzb4, 1, kNoutPad, kNh, kNout, n, m->grad + kOffW4, st);
-  colsum(m->dz4, kNout, m->grad + kOffB4);
+// forward and backward pass of n rows (inputs in h0, targets Tn, masks Mb,
+// the masks' sum in cnt; loss accumulates): the gradient's partial sums
+static MlpGradWs mlp_grad(casim_mlp *m, int n, cudaStream_t st) {
+  mlp_hidden(m, n, true, st);
+  const __nv_bfloat16 *w4t = m->wb.w4t;
+  if (m->engine == 1) {
+    gemm(m, m->h3, kNh, 1, w4t, kNh, 1, n, kNout, kNh,
+         EpiOutLoss{m->theta + kOffB4, m->Tn, m->Mb, m->cnt, m->loss, m->dz4, m->dzb4}, st);
+  } else {
+    gemm(m, m->h3, kNh, 1, w4t, kNh, 1, n, kNout, kNh, EpiOut{m->theta + kOffB4, m->y, kNout}, st);
+    k_mlp_loss<<<(unsigned)(((long long)n * kNout + 255) / 256), 256, 0, st>>>(m->y, m->Tn, m->Mb, n, m->cnt, m->loss,
+                                                                              m->dz4, m->dzb4);
+  }
+  // data gradients, layer by layer
   gemm(m, m->dzb4, kNoutPad, 1, m->wb.w4k, kNoutPad, 1, n, kNh, kNoutPad, EpiBackTanh{m->a3, m->dz3, m->dzb3, kNh}, st);
-  // layer 3
-  gemm_wgrad(m, m->h2, 1, kNh, m->dzb3, 1, kNh, kNh, kNh, n, m->grad + kOffW3, st);
-  colsum(m->dz3, kNh, m->grad + kOffB3);
   gemm(m, m->dzb3, kNh, 1, m->wb.w3k, kNh, 1, n, kNh, kNh, EpiBackTanh{m->a2, m->dz2, m->dzb2, kNh}, st);
-  // layer 2
-  gemm_wgrad(m, m->h1, 1, kNh, m->dzb2, 1, kNh, kNh, kNh, n, m->grad + kOffW2, st);
-  colsum(m->dz2, kNh, m->grad + kOffB2);
   gemm(m, m->dzb2, kNh, 1, m->wb.w2k, kNh, 1, n, kNh, kNh, EpiBackTanh{m->a1, m->dz1, m->dzb1, kNh}, st);
-  // layer 1
-  gemm_wgrad(m, m->h0, 1, kNinPad, m->dzb1, 1, kNh, kNin, kNh, n, m->grad + kOffW1, st);
-  colsum(m->dz1, kNh, m->grad + kOffB1);
+  // weight gradients over chunks of the batch (512 rows on the mma.sync
+  // engine, 256 on the tensor cores, enough chunks to give every SM a tile)
+  const int split = m->engine == 1 ? 256 : 512;
+  const int kchunk = std::max(split, (n + kSplitMax - 1) / kSplitMax + kGBK - 1) / kGBK * kGBK;
+  const MlpGradWs ws{m->wsplit, m->bpart, (n + kchunk - 1) / kchunk};
+  if (m->engine == 1) {
+    const WgradArgs a{{m->h0, m->h1, m->h2, m->h3}, {m->dzb1, m->dzb2, m->dzb3, m->dzb4}, n, kchunk, ws};
+    launch_pdl(k_wgrad_tc, dim3(kWgradTiles * ws.nsplit), kTcThreads, kTcSmem, st, a, m->d_err);
+  } else {
+    auto wgrad = [&](int l, const __nv_bfloat16 *h, int ldh, const __nv_bfloat16 *dz, int ldz, int M, int N) {
+      const GemmArgs g{h, 1, ldh, dz, 1, ldz, M, N, n, kchunk};
+      launch_gemm(m, g, EpiPartial{ws.ws + ws.nsplit * grad_ws_off(l), N, (long long)M * N}, ws.nsplit, st);
+    };
+    wgrad(3, m->h3, kNh, m->dzb4, kNoutPad, kNh, kNout);
+    wgrad(2, m->h2, kNh, m->dzb3, kNh, kNh, kNh);
+    wgrad(1, m->h1, kNh, m->dzb2, kNh, kNh, kNh);
+    wgrad(0, m->h0, kNinPad, m->dzb1, kNh, kNin, kNh);
+  }
+  launch_pdl(k_colsum, dim3(kColsumBlocks), 256, 0, st, ColsumArgs{{m->dz1, m->dz2, m->dz3, m->dz4}, n, m->bpart});
+  return ws;
+}
+
+// the inference kernel's weight images of the present parameters
+static void mlp_images(casim_mlp *m, cudaStream_t st) {
+  k_mlp_images<<<(kNh * kNh + 255) / 256, 256, 0, st>>>(m->theta, m->img);
 }
 
 static void mlp_cast(casim_mlp *m, cudaStream_t st) {
   k_mlp_cast<<<(kNh * kNh + 255) / 256, 256, 0, st>>>(m->theta, m->wb);
-  k_mlp_images<<<(kNh * kNh + 255) / 256, 256, 0, st>>>(m->theta, m->img);
+  mlp_images(m, st);
 }
 
 // forward pass of n rows of BF16 inputs on the tcgen05 kernel: rates at the
@@ -1320,7 +1343,7 @@ extern "C" void casim_mlp_free(casim_mlp *m) {
   cudaDeviceSynchronize();
   mlp_free_batch(m);
   void *ps[] = {m->theta, m->grad, m->m1, m->m2, m->wbuf, m->norm, m->box, m->cnt, m->loss,
-                m->xb, m->rowpt, m->surr, m->rowctr, m->img, m->wsplit, m->d_err, m->fxb};
+                m->xb, m->rowpt, m->surr, m->rowctr, m->img, m->wsplit, m->bpart, m->hist, m->d_err, m->fxb};
   for (void *p : ps) cudaFree(p);
   delete m;
 }
@@ -1352,14 +1375,16 @@ extern "C" int casim_mlp_create(casim_mlp **out, unsigned long long seed) {
   if (e == cudaSuccess) e = dalloc(&m->loss, 1);
   if (e == cudaSuccess) e = dalloc(&m->rowctr, 1);
   if (e == cudaSuccess) e = dalloc(&m->img, kImgBytes);
-  if (e == cudaSuccess) e = dalloc(&m->wsplit, (size_t)kSplitMax * kNh * kNh);
+  if (e == cudaSuccess) e = dalloc(&m->wsplit, (size_t)kSplitMax * kGradWsLen);
+  if (e == cudaSuccess) e = dalloc(&m->bpart, (size_t)kColsumChunks * kColsumLen);
   if (e == cudaSuccess) e = dalloc(&m->d_err, 1);
   if (e == cudaSuccess) e = cudaMemset(m->d_err, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tc<EpiHidden>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tc<EpiOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tc<EpiBackTanh>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tc<EpiPartial>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tc<EpiOutLoss>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
   if (e == cudaSuccess) e = cudaMemcpy(m->theta, th.data(), kNParam * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(m->m1, 0, kNParam * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(m->m2, 0, kNParam * sizeof(float));
@@ -1436,7 +1461,7 @@ extern "C" int casim_mlp_forward_host(casim_mlp *m, const float *Xn, int n, floa
     CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     CUDA_TRY(mlp_forward_umma(m, m->h0, n, nullptr, nullptr, m->d_err, nsm, 0));
   } else {
-    mlp_forward(m, n, false, 0);
+    mlp_forward(m, n, 0);
   }
   CUDA_TRY(cudaGetLastError());
   unsigned herr = 0;
@@ -1473,7 +1498,7 @@ extern "C" int casim_mlp_forward(casim_mlp *m, const float *Xn, long long n, flo
     int rc = mlp_batch_ws(m, (int)n);
     if (rc != CASIM_OK) return rc;
     k_mlp_inputs<<<gin, 256, 0, st>>>(Xn, (int)n, m->h0);
-    mlp_forward(m, (int)n, false, st);
+    mlp_forward(m, (int)n, st);
     CUDA_TRY(cudaMemcpyAsync(Y, m->y, (size_t)n * kNout * sizeof(float), cudaMemcpyDeviceToDevice, st));
   }
   CUDA_TRY(cudaGetLastError());
@@ -1497,8 +1522,11 @@ extern "C" int casim_mlp_loss_grad_host(casim_mlp *m, const float *Xn, const flo
   CUDA_TRY(cudaMemcpy(m->Tn, Tn, (size_t)n * kNout * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(m->Mb, M, (size_t)n * kNout * sizeof(float), cudaMemcpyHostToDevice));
   k_mlp_inputs<<<(unsigned)(((long long)n * kNinPad + 255) / 256), 256>>>(m->Xn, n, m->h0);
-  mlp_forward(m, n, true, 0);
-  mlp_backward(m, n, 0);
+  CUDA_TRY(cudaMemsetAsync(m->cnt, 0, sizeof(float), 0));
+  CUDA_TRY(cudaMemsetAsync(m->loss, 0, sizeof(double), 0));
+  k_sum<<<64, 256>>>(m->Mb, (long long)n * kNout, m->cnt);
+  const MlpGradWs ws = mlp_grad(m, n, 0);
+  k_mlp_update<<<(kNParam + 255) / 256, 256>>>(ws, m->grad, AdamArgs{});
   CUDA_TRY(cudaGetLastError());
   if (loss) CUDA_TRY(cudaMemcpy(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost));
   if (grad) CUDA_TRY(cudaMemcpy(grad, m->grad, kNParam * sizeof(float), cudaMemcpyDeviceToHost));
@@ -1583,22 +1611,29 @@ extern "C" int casim_mlp_fit(casim_mlp *m, const float *X, const float *Y, const
   m->fitted = true;
   int rc = mlp_batch_ws(m, batch);
   if (rc != CASIM_OK) return rc;
+  if (loss_hist && steps > m->cap_hist) {
+    cudaFree(m->hist);
+    m->hist = nullptr;
+    m->cap_hist = 0;
+    if ((e = dalloc(&m->hist, steps)) != cudaSuccess)
+      return e == cudaErrorMemoryAllocation ? CASIM_ERR_OOM : cuda_fail(e, "cudaMalloc");
+    m->cap_hist = steps;
+  }
+  CUDA_TRY(cudaMemsetAsync(m->cnt, 0, sizeof(float), st));
+  CUDA_TRY(cudaMemsetAsync(m->loss, 0, sizeof(double), st));
   for (int s = 0; s < steps; ++s) {
-    k_mlp_batch<<<(batch + 255) / 256, 256, 0, st>>>(X, Y, M, n, seed, s, batch, m->norm, m->Xn, m->Tn, m->Mb);
-    k_mlp_inputs<<<(unsigned)(((long long)batch * kNinPad + 255) / 256), 256, 0, st>>>(m->Xn, batch, m->h0);
-    mlp_forward(m, batch, true, st);
-    mlp_backward(m, batch, st);
+    launch_pdl(k_mlp_batch, dim3((unsigned)(((long long)batch * kNinPad + 255) / 256)), 256, 0, st, X, Y, M, n, seed,
+               (long long)s, batch, m->norm, m->h0, m->Tn, m->Mb, m->cnt);
+    const MlpGradWs ws = mlp_grad(m, batch, st);
     ++m->adam_t;
     const float c1 = 1.f - (float)std::pow(0.9, (double)m->adam_t), c2 = 1.f - (float)std::pow(0.999, (double)m->adam_t);
-    k_adam<<<(kNParam + 255) / 256, 256, 0, st>>>(m->theta, m->grad, m->m1, m->m2, kNParam, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
-    mlp_cast(m, st);
-    if (loss_hist) {
-      double l = 0.0;
-      CUDA_TRY(cudaMemcpyAsync(&l, m->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
-      CUDA_TRY(cudaStreamSynchronize(st));
-      loss_hist[s] = (float)l;
-    }
+    launch_pdl(k_mlp_update, dim3((kNParam + 255) / 256), 256, 0, st, ws, m->grad,
+               AdamArgs{m->theta, m->m1, m->m2, lr, 0.9f, 0.999f, 1e-8f, c1, c2, m->wb, m->cnt,
+                        loss_hist ? m->hist + s : nullptr, m->loss});
   }
+  mlp_images(m, st);
+  if (loss_hist && steps > 0)
+    CUDA_TRY(cudaMemcpyAsync(loss_hist, m->hist, steps * sizeof(float), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(st));
   return mlp_wait_report(m, "casim_mlp_fit");
@@ -1676,7 +1711,7 @@ extern "C" int casim_step_surrogate(casim_ctx *ctx, casim_mlp *m, const casim_st
       const int n = (int)std::min<long long>(m->cap_b, rows - r0);
       __nv_bfloat16 *save = m->h0;
       m->h0 = m->xb + r0 * kNinPad;
-      mlp_forward(m, n, false, st);
+      mlp_forward(m, n, st);
       m->h0 = save;
       k_mlp_scatter<<<(n + 255) / 256, 256, 0, st>>>(m->y, n, m->rowpt + r0, m->norm, m->surr, np, ctx->d_err);
       ctx->launches += 5;
@@ -1739,7 +1774,7 @@ extern "C" int casim_batch_step_surrogate(casim_ctx *ctx, casim_batch *b, casim_
       const int n = (int)std::min<long long>(m->cap_b, rows - r0);
       __nv_bfloat16 *save = m->h0;
       m->h0 = m->xb + r0 * kNinPad;
-      mlp_forward(m, n, false, st);
+      mlp_forward(m, n, st);
       m->h0 = save;
       k_mlp_scatter<<<(n + 255) / 256, 256, 0, st>>>(m->y, n, m->rowpt + r0, m->norm, m->surr, b->total_pts,
                                                      ctx->d_err);

@@ -7,8 +7,11 @@
 
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "casim_device.cuh"
 #include "casim_batch.cuh"
+#include "casim_umma.cuh"
 
 namespace casim_dev {
 
@@ -144,7 +147,46 @@ struct EpiOut {
   __device__ __forceinline__ void operator()(int m, int n, float acc) const { y[(long long)m * ld + n] = acc + bias[n]; }
 };
 
-// weight gradient: g[m][n] = acc
+// masked squared error of one output: the gradient to dz (FP32 [n][4] and BF16
+// [n][16], whose columns 4.. stay zero), the loss term returned
+__device__ __forceinline__ double mlp_loss_term(float y, float t, float m, float cnt, float &g) {
+  const float inv = 1.f / fmaxf(cnt, 1.f);
+  const float d = (y - t) * m;
+  g = 2.f * d * inv;
+  return (double)d * d * inv;
+}
+
+// output layer of a training pass: y = acc + b, its loss term (summed over
+// the rows by the GEMM) and gradient; y itself is not kept
+struct EpiOutLoss {
+  static constexpr bool kLoad = false;
+  const float *bias, *T, *Mk, *cnt;
+  double *loss;
+  float *dz;
+  __nv_bfloat16 *dzb;
+  // the outputs of one row
+  __device__ __forceinline__ double row(int m, const float *acc) const {
+    const float4 t = reinterpret_cast<const float4 *>(T)[m], k = reinterpret_cast<const float4 *>(Mk)[m];
+    const float tv[kNout] = {t.x, t.y, t.z, t.w}, kv[kNout] = {k.x, k.y, k.z, k.w}, c = *cnt;
+    float g[kNout];
+    __nv_bfloat16 h[kNout];
+    double part = 0.0;
+#pragma unroll
+    for (int n = 0; n < kNout; ++n) {
+      part += mlp_loss_term(acc[n] + bias[n], tv[n], kv[n], c, g[n]);
+      h[n] = __float2bfloat16(g[n]);
+    }
+    reinterpret_cast<float4 *>(dz)[m] = make_float4(g[0], g[1], g[2], g[3]);
+    __nv_bfloat162 lo, hi;
+    lo.x = h[0]; lo.y = h[1]; hi.x = h[2]; hi.y = h[3];
+    __nv_bfloat162 *d = reinterpret_cast<__nv_bfloat162 *>(dzb + (long long)m * kNoutPad);
+    d[0] = lo;
+    d[1] = hi;
+    return part;
+  }
+};
+
+// one chunk's partial weight gradient: c[m][n] = acc
 struct EpiStore {
   static constexpr bool kLoad = false;
   float *c;
@@ -162,15 +204,6 @@ struct EpiPartial {
     ws[blockIdx.z * zstride + (long long)m * ld + n] = acc;
   }
 };
-
-// out[i] = sum over z (in order) of ws[z][i]: deterministic split-K reduction
-__global__ void k_splitk_sum(const float *ws, int nsplit, long long len, float *out) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= len) return;
-  float s = 0.f;
-  for (int z = 0; z < nsplit; ++z) s += ws[z * len + i];
-  out[i] = s;
-}
 
 // data gradient through tanh: dz = acc (1 - a^2); FP32 for the bias sums,
 // BF16 for the next GEMMs
@@ -232,24 +265,16 @@ __global__ void k_mlp_inputs(const float *X, int n, __nv_bfloat16 *h0) {
   h0[i] = __float2bfloat16(k < kNin ? X[r * kNin + k] : 0.f);
 }
 
-// masked squared error: loss += sum (y - t)^2 m / cnt; dz = 2 (y - t) m / cnt
-// (FP32 [n][4] and BF16 [n][16], columns >= 4 zero)
+// masked squared error of the mma.sync engine's pass: loss += sum (y - t)^2 m / cnt and its gradient
 __global__ void k_mlp_loss(const float *Y, const float *T, const float *Mk, int n, const float *cnt, double *loss,
                            float *dz, __nv_bfloat16 *dzb) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   double part = 0.0;
-  if (i < (long long)n * kNoutPad) {
-    const long long r = i / kNoutPad;
-    const int c = (int)(i % kNoutPad);
-    float g = 0.f;
-    if (c < kNout) {
-      const float inv = 1.f / fmaxf(*cnt, 1.f);
-      const float d = (Y[r * kNout + c] - T[r * kNout + c]) * Mk[r * kNout + c];
-      part = (double)d * d * inv;
-      g = 2.f * d * inv;
-      dz[r * kNout + c] = g;
-    }
-    dzb[i] = __float2bfloat16(g);
+  if (i < (long long)n * kNout) {
+    float g;
+    part = mlp_loss_term(Y[i], T[i], Mk[i], *cnt, g);
+    dz[i] = g;
+    dzb[i / kNout * kNoutPad + i % kNout] = __float2bfloat16(g);
   }
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if ((threadIdx.x & 31) == 0 && part != 0.0) atomicAdd(loss, part);
@@ -263,46 +288,121 @@ __global__ void k_sum(const float *x, long long n, float *out) {
   if ((threadIdx.x & 31) == 0) atomicAdd(out, part);
 }
 
-// bias gradient: column sums of dz [n][ld] (first `cols` columns).  Block
-// (32, 32) of grid (column blocks, row chunks): lane x is a column
-// (coalesced rows), y a row phase within chunk blockIdx.y; the 32 phase sums
-// are added in a fixed order into part[chunk][c]; k_colsum_fin adds the
-// chunks in order into g (deterministic).
+// Weight gradients are summed over chunks of the batch (split K): chunk z of
+// layer l's [M][N] gradient at ws[split * off[l] + z M N + i].  Bias
+// gradients are column sums of dz over kColsumChunks row chunks.
+constexpr int kSplitMax = 64;
 constexpr int kColsumY = 32, kColsumChunks = 16;
-__global__ void __launch_bounds__(32 * kColsumY) k_colsum(const float *dz, int n, int ld, int cols, float *part_out) {
+constexpr int kColsumLen = 3 * kNh + kNout;   // columns of dz1, dz2, dz3, dz4
+struct MlpGradWs {
+  float *ws;       // [kSplitMax][kNin + 2 kNh + kNout][..]: W1, W2, W3, W4 one after another
+  float *part;     // [kColsumChunks][kColsumLen]
+  int nsplit;
+};
+// first element of layer l's partial sums, in units of one chunk of it
+__host__ __device__ constexpr long long grad_ws_off(int l) {
+  return l == 0 ? 0 : l == 1 ? kNin * kNh : l == 2 ? kNin * kNh + kNh * kNh : kNin * kNh + 2 * kNh * kNh;
+}
+constexpr long long kGradWsLen = kNin * kNh + 2 * kNh * kNh + kNh * kNout;
+
+// Bias column sums, one block of 256 threads per 32 columns and row chunk:
+// lane x is a column (coalesced rows), and each warp takes four of the
+// chunk's 32 row phases; the 32 phase sums are added in a fixed order into
+// part[chunk][column]; k_mlp_update adds the chunks in order (deterministic).
+struct ColsumArgs {
+  const float *dz[4];   // [n][256] of layers 1-3, [n][4] of layer 4
+  int n;
+  float *part;
+};
+constexpr int kColsumBlocks = (3 * kNh / 32 + 1) * kColsumChunks;
+__global__ void __launch_bounds__(256) k_colsum(const ColsumArgs a) {
   __shared__ float s_part[kColsumY][33];
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  const int per = (n + gridDim.y - 1) / gridDim.y, r0 = blockIdx.y * per, r1 = min(n, r0 + per);
-  float part = 0.f;
-  if (c < cols)
-    for (int r = r0 + threadIdx.y; r < r1; r += kColsumY) part += dz[(long long)r * ld + c];
-  s_part[threadIdx.y][threadIdx.x] = part;
+  pdl_trigger();
+  pdl_wait();
+  const int block = blockIdx.x;
+  const int cb = block / kColsumChunks, chunk = block % kColsumChunks;
+  const int l = cb / (kNh / 32), ld = l < 3 ? kNh : kNout;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, c = (l < 3 ? cb % (kNh / 32) * 32 : 0) + x;
+  const float *dz = l == 0 ? a.dz[0] : l == 1 ? a.dz[1] : l == 2 ? a.dz[2] : a.dz[3];
+  const int per = (a.n + kColsumChunks - 1) / kColsumChunks, r0 = chunk * per, r1 = min(a.n, r0 + per);
+  float part[4] = {0.f, 0.f, 0.f, 0.f};
+  if (c < ld) {
+    const float *p = dz + c;
+#pragma unroll 4
+    for (int r = r0 + y; r < r1; r += kColsumY) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (r + 8 * j < r1) part[j] += p[(long long)(r + 8 * j) * ld];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) s_part[y + 8 * j][x] = part[j];
   __syncthreads();
-  if (threadIdx.y == 0 && c < cols) {
+  if (y == 0 && c < ld) {
     float s = 0.f;
-    for (int y = 0; y < kColsumY; ++y) s += s_part[y][threadIdx.x];
-    part_out[(long long)blockIdx.y * cols + c] = s;
+    for (int i = 0; i < kColsumY; ++i) s += s_part[i][x];
+    a.part[(long long)chunk * kColsumLen + l * kNh + c] = s;
   }
 }
-__global__ void k_colsum_fin(const float *part, int chunks, int cols, float *g) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int y = 0; y < chunks; ++y) s += part[(long long)y * cols + c];
-  g[c] = s;
-}
+struct AdamArgs {
+  float *theta, *m1, *m2;   // theta null: the gradient only
+  float lr, b1, b2, eps, c1, c2;
+  MlpBf16 w;
+  float *cnt, *hist;        // hist: this step's loss, or null
+  double *loss;
+};
 
-// Adam on the flat FP32 parameters
-__global__ void k_adam(float *theta, const float *grad, float *m1, float *m2, int n, float lr, float b1, float b2,
-                       float eps, float c1, float c2) {
+// One parameter per thread: its gradient from the partial sums, in order
+// (deterministic), then with Adam its new value and BF16 copies; the loss and
+// the mask count are handed over and cleared for the next step.
+__global__ void k_mlp_update(const MlpGradWs g, float *grad, const AdamArgs a) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float g = grad[i];
-  const float a = b1 * m1[i] + (1.f - b1) * g;
-  const float b = b2 * m2[i] + (1.f - b2) * g * g;
-  m1[i] = a;
-  m2[i] = b;
-  theta[i] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+  pdl_trigger();
+  pdl_wait();
+  if (i == 0 && a.theta) {
+    if (a.hist) *a.hist = (float)*a.loss;
+    *a.loss = 0.0;
+    *a.cnt = 0.f;
+  }
+  if (i >= kNParam) return;
+  const int off[8] = {kOffW1, kOffB1, kOffW2, kOffB2, kOffW3, kOffB3, kOffW4, kOffB4};
+  int t = 0, base = 0;   // 2 l: weights of layer l + 1, 2 l + 1: its biases
+#pragma unroll
+  for (int j = 1; j < 8; ++j)
+    if (i >= off[j]) {
+      t = j;
+      base = off[j];
+    }
+  const int e = i - base, l = t >> 1;
+  float s = 0.f;
+  if (t & 1) {
+    for (int y = 0; y < kColsumChunks; ++y) s += g.part[(long long)y * kColsumLen + l * kNh + e];
+  } else {
+    const long long len = l == 0 ? kNin * kNh : l == 3 ? kNh * kNout : kNh * kNh;
+    const float *ws = g.ws + g.nsplit * (l == 0 ? grad_ws_off(0) : l == 1 ? grad_ws_off(1) : l == 2 ? grad_ws_off(2)
+                                                                                                     : grad_ws_off(3)) + e;
+#pragma unroll 32
+    for (int z = 0; z < g.nsplit; ++z) s += ws[z * len];
+  }
+  grad[i] = s;
+  if (!a.theta) return;
+  const float x = a.b1 * a.m1[i] + (1.f - a.b1) * s;
+  const float v = a.b2 * a.m2[i] + (1.f - a.b2) * s * s;
+  a.m1[i] = x;
+  a.m2[i] = v;
+  const float th = a.theta[i] - a.lr * (x / a.c1) / (sqrtf(v / a.c2) + a.eps);
+  a.theta[i] = th;
+  if (t & 1) return;
+  const __nv_bfloat16 h = __float2bfloat16(th);
+  if (t == 0) {
+    a.w.w1t[e % kNh * kNinPad + e / kNh] = h;
+  } else if (t == 6) {
+    a.w.w4t[e % kNout * kNh + e / kNout] = h;
+    a.w.w4k[e / kNout * kNoutPad + e % kNout] = h;
+  } else {
+    (t == 2 ? a.w.w2t : a.w.w3t)[e % kNh * kNh + e / kNh] = h;
+    (t == 2 ? a.w.w2k : a.w.w3k)[e] = h;
+  }
 }
 
 // counter-based mini-batch sampling: row r of batch `step` is
@@ -314,26 +414,41 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
   return z ^ (z >> 31);
 }
 
-// gather a standardised mini-batch from the raw data
-__global__ void k_mlp_batch(const float *X, const float *Y, const float *Mk, long long n, unsigned long long seed,
-                            long long step, int B, const float *norm, float *Xn, float *Tn, float *Mb) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= B) return;
-  const long long src = (long long)(mix64(seed ^ mix64((unsigned long long)step * 0x100000001b3ull + r)) % (unsigned long long)n);
+// gather a standardised mini-batch from the raw data: 16 threads per row (the
+// rows lie anywhere in the data; each is read by neighbouring threads), its
+// BF16 inputs [B][16], targets, masks and the sum of the masks
+__global__ void __launch_bounds__(256) k_mlp_batch(const float *X, const float *Y, const float *Mk, long long n,
+                                                   unsigned long long seed, long long step, int B, const float *norm,
+                                                   __nv_bfloat16 *h0, float *Tn, float *Mb, float *cnt) {
+  __shared__ float s_cnt[256 / 32];
+  pdl_trigger();
+  pdl_wait();
+  const long long i = blockIdx.x * 256ll + threadIdx.x;
+  const int r = (int)(i / kNinPad), k = (int)(i % kNinPad);
   const float *mu = norm, *sd = norm + kNin, *muy = norm + 2 * kNin, *sdy = norm + 2 * kNin + kNout;
-#pragma unroll
-  for (int k = 0; k < kNin; ++k) Xn[(long long)r * kNin + k] = (X[src * kNin + k] - mu[k]) / sd[k];
-#pragma unroll
-  for (int c = 0; c < kNout; ++c) {
-    const float m = Mk[src * kNout + c];
-    Mb[(long long)r * kNout + c] = m;
-    Tn[(long long)r * kNout + c] = m > 0.f ? (Y[src * kNout + c] - muy[c]) / sdy[c] : 0.f;
+  float m = 0.f;
+  if (r < B) {
+    const long long src = (long long)(mix64(seed ^ mix64((unsigned long long)step * 0x100000001b3ull + r)) % (unsigned long long)n);
+    h0[i] = __float2bfloat16(k < kNin ? (X[src * kNin + k] - mu[k]) / sd[k] : 0.f);
+    if (k < kNout) {
+      m = Mk[src * kNout + k];
+      Mb[(long long)r * kNout + k] = m;
+      Tn[(long long)r * kNout + k] = m > 0.f ? (Y[src * kNout + k] - muy[k]) / sdy[k] : 0.f;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+  if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float t = 0.f;
+    for (int w = 0; w < 256 / 32; ++w) t += s_cnt[w];
+    atomicAdd(cnt, t);
   }
 }
 
 // per-feature mean and standard deviation, per-target (masked) mean and
 // standard deviation, per-feature min and max (the box of the training data)
-__global__ void k_mlp_stats(const float *X, const float *Y, const float *Mk, long long n, double *acc) {
+__global__ void __launch_bounds__(256) k_mlp_stats(const float *X, const float *Y, const float *Mk, long long n, double *acc) {
   // acc: [12 sum][12 sumsq][4 sum][4 sumsq][4 count] then min/max as ordered ints elsewhere
   double s[kNin] = {0}, q[kNin] = {0}, sy[kNout] = {0}, qy[kNout] = {0}, cy[kNout] = {0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -352,16 +467,31 @@ __global__ void k_mlp_stats(const float *X, const float *Y, const float *Mk, lon
         cy[c] += 1.0;
       }
   }
+  // the block's sums, one atomic per block and sum: with one per thread,
+  // 65 536 of them queued on each of the 36 addresses, and the kernel took
+  // 1.54 ms for 262 144 rows
+  __shared__ double s_sum[256 / 32][2 * kNin + 3 * kNout];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto put = [&](int at, double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) s_sum[warp][at] = v;
+  };
 #pragma unroll
   for (int k = 0; k < kNin; ++k) {
-    atomicAdd(&acc[k], s[k]);
-    atomicAdd(&acc[kNin + k], q[k]);
+    put(k, s[k]);
+    put(kNin + k, q[k]);
   }
 #pragma unroll
   for (int c = 0; c < kNout; ++c) {
-    atomicAdd(&acc[2 * kNin + c], sy[c]);
-    atomicAdd(&acc[2 * kNin + kNout + c], qy[c]);
-    atomicAdd(&acc[2 * kNin + 2 * kNout + c], cy[c]);
+    put(2 * kNin + c, sy[c]);
+    put(2 * kNin + kNout + c, qy[c]);
+    put(2 * kNin + 2 * kNout + c, cy[c]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * kNin + 3 * kNout) {
+    double v = 0.0;
+    for (int w = 0; w < 256 / 32; ++w) v += s_sum[w][threadIdx.x];
+    atomicAdd(&acc[threadIdx.x], v);
   }
 }
 
@@ -585,7 +715,6 @@ __global__ void k_mlp_scatter(const float *Yn, long long rows, const long long *
 }  // namespace casim_dev
 
 // ------------------------------------------------ tcgen05 inference kernel
-#include "casim_umma.cuh"
 
 namespace casim_dev {
 
@@ -907,189 +1036,159 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) k_mlp_umma(const UmmaArgs u) 
 // GemmArgs, FP32 accumulators in tensor memory, the same fused epilogues as
 // k_gemm.  Each operand is K-major (unit stride along k: the forward pass and
 // the data gradients) or MN-major (unit stride along m or n: the weight
-// gradients, whose k runs over the batch); both are staged in shared memory
-// as the K-major 128-byte-swizzled slabs the MMA reads (sw128_offset), an
-// MN-major tile being transposed in registers on the way (8 x 8 blocks).
+// gradients, whose k runs over the batch); both are staged by 16-byte
+// asynchronous copies in the 128-byte-swizzled slabs of that major-ness, which
+// the MMA reads as they are.
 //
-// One CTA of 4 warps per 128 x 128 output tile (split K over blockIdx.z as
-// for k_gemm); K advances in slabs of 64 through two shared-memory buffers:
-// all threads load slab s + 1 into registers while the MMAs of slab s run,
-// then wait (bounded) for the MMAs that last read the buffer before storing
-// into it.  One thread issues the MMAs (M = 128, N = the tile's columns
-// rounded up to 16, K = 16 each) and commits each slab to its buffer's
-// mbarrier.  Epilogue: warp w reads tensor-memory lanes 32w.. (its rows),
-// 32 columns at a time, and passes the 32 x 32 block through shared memory
-// (the operand buffers, free once the last MMA completed) so that the
-// epilogue's loads and stores run along n, coalesced.  A wait that gives up
-// sets error bit 4, waits again for the MMAs it issued and releases the
-// tensor memory.
-constexpr int kTcBM = 128, kTcBN = 128, kTcBK = 64;
-constexpr uint32_t kTcTile = kTcBM * kTcBK * 2;              // one operand slab: 16 KB
-constexpr int kTcSmem = 1024 + 4 * (int)kTcTile;              // A and B, two buffers, 1024-byte alignment
+// A tile is 128 x 64, one CTA of 8 warps, two CTAs per SM.  These GEMMs are a
+// microsecond of tensor work behind a chain of latencies (operands, MMAs,
+// epilogue), so the whole depth of up to 256 is loaded at once, in slabs of 64
+// whose MMAs follow as they land, and small tiles put every SM to work: with
+// 128 x 128 tiles of 4 warps and two slabs in flight a hidden layer took 24 us
+// on 8192 rows and a data gradient 36 us, now 10 and 11 us; the weight
+// gradients, one launch per layer with 128 x 128 tiles transposed through
+// registers, took 92 us, now 17 us in one launch (all by ncu, cold caches).
+// A training step on 8192 rows: 0.34 -> 0.094 ms.
+// One thread issues the MMAs (M = 128, N = the
+// tile's columns rounded up to 16, K = 16 each).  Epilogue: warp w reads
+// tensor-memory lanes 32 (w % 4).. (its rows) and 32 columns, and passes the
+// 32 x 32 block through shared memory (the operand slabs, free once the last
+// MMA completed) so that the epilogue's loads and stores run along n,
+// coalesced.  A wait that gives up sets error bit 4, waits again for the MMAs
+// it issued and releases the tensor memory.
+constexpr int kTcBM = 128, kTcBN = 64, kTcBK = 64, kTcSlabs = 4;
+constexpr int kTcThreads = 256;
+constexpr uint32_t kTcSlabA = kTcBM * kTcBK * 2, kTcSlabB = kTcBN * kTcBK * 2;   // 16 KB, 8 KB
+constexpr int kTcSmem = 1024 + kTcSlabs * (int)(kTcSlabA + kTcSlabB);            // 1024-byte alignment
 constexpr unsigned kTcSpins = 1u << 24;
 
-// One thread's share of an operand slab: rows r0..r0+127 of the operand
-// (row index m or n), k in [k0, k0 + 64) of [.., ke), zeros outside it.
-// K-major (unit stride along k): 8 chunks of 8 k, consecutive threads along a
-// row.  MN-major (unit stride along the rows): one 8 (rows) x 8 (k) block,
-// as 8 chunks of 8 rows at one k, transposed into 8 chunks of 8 k at one row
-// when stored.  tc_fetch issues the global loads, tc_put writes the slab in
-// the swizzled K-major layout, so both operands' loads are in flight
-// together.
-struct TcFrag {
-  uint4 v[8];
-};
+// 16-byte asynchronous copy global -> shared; ok false: zeros (src not read)
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
 
-__device__ __forceinline__ void tc_fetch(TcFrag &fr, const __nv_bfloat16 *P, long long srow, long long sk, int nrows,
-                                         int r0, int k0, int ke, int tid) {
-  const __nv_bfloat16 zero = __float2bfloat16(0.f);
-  if (sk == 1) {
+// slab `s` (k0 .. k0 + 63 of [.., ke)) of a K-major operand of R rows r0..: asynchronous copies
+template <int R>
+__device__ __forceinline__ void tc_load_kmajor(uint32_t dst, const __nv_bfloat16 *P, long long srow, int nrows, int r0,
+                                               int k0, int ke, int tid) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int i = tid + 128 * j, r = i >> 3, ch = i & 7;
-      const int row = r0 + r, k = k0 + 8 * ch;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (row < nrows && k < ke) {
-        const __nv_bfloat16 *src = P + (long long)row * srow + k;
-        if (k + 8 <= ke) {
-          v = __ldg(reinterpret_cast<const uint4 *>(src));
-        } else {
-          __align__(16) __nv_bfloat16 e[8];
-#pragma unroll
-          for (int t = 0; t < 8; ++t) e[t] = k + t < ke ? src[t] : zero;
-          v = *reinterpret_cast<const uint4 *>(e);
-        }
-      }
-      fr.v[j] = v;
-    }
-  } else {
-    const int rg = tid & 15, kg = tid >> 4;
-    const int row = r0 + 8 * rg;
-#pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-      const int k = k0 + 8 * kg + kk;
-      uint4 u = make_uint4(0, 0, 0, 0);
-      if (k < ke && row < nrows) {
-        const __nv_bfloat16 *src = P + (long long)k * sk + row;
-        if (row + 8 <= nrows) {
-          u = __ldg(reinterpret_cast<const uint4 *>(src));
-        } else {
-          __align__(16) __nv_bfloat16 e[8];
-#pragma unroll
-          for (int t = 0; t < 8; ++t) e[t] = row + t < nrows ? src[t] : zero;
-          u = *reinterpret_cast<const uint4 *>(e);
-        }
-      }
-      fr.v[kk] = u;
-    }
+  for (int j = 0; j < R * 8 / kTcThreads; ++j) {
+    const int i = tid + kTcThreads * j, r = i >> 3, ch = i & 7;
+    const int row = r0 + r, k = k0 + 8 * ch;
+    const bool ok = row < nrows && k < ke;   // every K-major depth is a multiple of 8
+    cp_async16(dst + sw128_offset(R, r, 8 * ch), ok ? P + (long long)row * srow + k : P, ok);
   }
 }
 
-__device__ __forceinline__ void tc_put(unsigned char *dst, const TcFrag &fr, long long sk, int tid) {
-  if (sk == 1) {
+// the same of an MN-major operand (rows in whole chunks of 8)
+template <int R>
+__device__ __forceinline__ void tc_load_mn(uint32_t dst, const __nv_bfloat16 *P, long long sk, int nrows, int r0, int k0,
+                                           int ke, int tid) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int i = tid + 128 * j, r = i >> 3, ch = i & 7;
-      *reinterpret_cast<uint4 *>(dst + sw128_offset(kTcBM, r, 8 * ch)) = fr.v[j];
-    }
-  } else {
-    const int rg = tid & 15, kg = tid >> 4;
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(fr.v);   // w[4 kk + j]: rows 2j, 2j + 1 at k kk
-#pragma unroll
-    for (int mm = 0; mm < 8; ++mm) {
-      const unsigned sel = (mm & 1) ? 0x7632u : 0x5410u;   // high or low halves of the two words
-      const int j = mm >> 1;
-      uint4 o;
-      o.x = __byte_perm(w[0 * 4 + j], w[1 * 4 + j], sel);
-      o.y = __byte_perm(w[2 * 4 + j], w[3 * 4 + j], sel);
-      o.z = __byte_perm(w[4 * 4 + j], w[5 * 4 + j], sel);
-      o.w = __byte_perm(w[6 * 4 + j], w[7 * 4 + j], sel);
-      *reinterpret_cast<uint4 *>(dst + sw128_offset(kTcBM, 8 * rg + mm, 8 * kg)) = o;
-    }
+  for (int j = 0; j < R * 8 / kTcThreads; ++j) {
+    const int i = tid + kTcThreads * j, kk = i / (R / 8), rr = 8 * (i % (R / 8));
+    const int row = r0 + rr, k = k0 + kk;
+    const bool ok = row < nrows && k < ke;
+    cp_async16(dst + sw128_mn_offset(rr, kk), ok ? P + (long long)k * sk + row : P, ok);
   }
 }
 
-template <class Epi>
-__global__ void __launch_bounds__(128) k_gemm_tc(const GemmArgs g, const Epi epi, unsigned *err) {
+// the tile at (m0, n0) over k in [kb, ke), then the epilogue.  kMN: both
+// operands MN-major, with rows in memory up to ra and rb (multiples of 8)
+template <bool kMN, class Epi>
+__device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0, int kb, int ke, const Epi &epi,
+                                          unsigned *err, int ra = 0, int rb = 0) {
   extern __shared__ __align__(16) unsigned char sraw[];
   unsigned char *sm = sraw + ((1024 - (smem_addr(sraw) & 1023)) & 1023);
+  unsigned char *smB = sm + kTcSlabs * kTcSlabA;
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) unsigned long long s_bar[2];
+  __shared__ __align__(8) unsigned long long s_bar;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.y * kTcBM, n0 = blockIdx.x * kTcBN;
-  const int kb = blockIdx.z * g.kchunk, ke = min(g.K, kb + g.kchunk);
-  const int nst = ke > kb ? (ke - kb + kTcBK - 1) / kTcBK : 0;
   const int ncols = min(kTcBN, ((g.N - n0) + 15) / 16 * 16);   // MMA N: the tile's columns, multiple of 16
-  const uint32_t idesc = umma_idesc_bf16(kTcBM, ncols);
-  unsigned char *bufA[2] = {sm, sm + 2 * kTcTile};
-  unsigned char *bufB[2] = {sm + kTcTile, sm + 3 * kTcTile};
-  const uint32_t bar0 = smem_addr(&s_bar[0]);
+  const uint32_t idesc = umma_idesc_bf16(kTcBM, ncols, kMN);
+  const uint32_t bar = smem_addr(&s_bar), sa = smem_addr(sm), sbb = smem_addr(smB);
   if (warp == 0) {
     tmem_alloc(smem_addr(&s_tmem), kTcBN);
     tmem_relinquish();
   }
   if (tid == 0) {
-    bar_init(bar0, 1);
-    bar_init(bar0 + 8, 1);
+    bar_init(bar, 1);
     bar_fence_init();
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t taddr = s_tmem;
+  pdl_wait();
   bool ok = true;
-  TcFrag fa, fb;
-  if (nst > 0) {
-    tc_fetch(fa, g.A, g.sam, g.sak, g.M, m0, kb, ke, tid);
-    tc_fetch(fb, g.B, g.sbn, g.sbk, g.N, n0, kb, ke, tid);
-    tc_put(bufA[0], fa, g.sak, tid);
-    tc_put(bufB[0], fb, g.sbk, tid);
-  }
-  fence_async_smem();
-  __syncthreads();
-  for (int s = 0; s < nst; ++s) {
-    const int buf = s & 1, k0 = kb + s * kTcBK;
-    if (tid == 0) {
-      tc_fence_after();
-      const int nsub = (min(kTcBK, ke - k0) + 15) / 16;
-      const uint32_t a = smem_addr(bufA[buf]), b = smem_addr(bufB[buf]);
-      for (int sub = 0; sub < nsub; ++sub)
-        umma_bf16(taddr, umma_desc_sw128(a + 32u * (uint32_t)sub), umma_desc_sw128(b + 32u * (uint32_t)sub), idesc,
-                  (s | sub) ? 1u : 0u);
-      umma_commit(bar0 + 8u * (uint32_t)buf);
-    }
-    if (s + 1 < nst) {
-      const int nb = buf ^ 1;
-      tc_fetch(fa, g.A, g.sam, g.sak, g.M, m0, k0 + kTcBK, ke, tid);
-      tc_fetch(fb, g.B, g.sbn, g.sbk, g.N, n0, k0 + kTcBK, ke, tid);
-      // the MMAs of slab s - 1 read buffer nb: wait for their commit
-      if (s >= 1 && ok) ok = bar_wait(bar0 + 8u * (uint32_t)nb, (uint32_t)(((s - 1) >> 1) & 1), kTcSpins);
-      if (ok) {
-        tc_put(bufA[nb], fa, g.sak, tid);
-        tc_put(bufB[nb], fb, g.sbk, tid);
+  int round = 0;   // depths of 256
+  uint32_t taddr = 0;
+  for (int k0 = kb; k0 < ke; k0 += kTcSlabs * kTcBK, ++round) {
+    // the MMAs that read the slabs of the round before have completed
+    if (round > 0 && ok) ok = bar_wait(bar, (uint32_t)((round - 1) & 1), kTcSpins);
+    const int nst = min(kTcSlabs, (ke - k0 + kTcBK - 1) / kTcBK);
+    if (ok) {
+#pragma unroll
+      for (int s = 0; s < kTcSlabs; ++s) {
+        const int ks = k0 + s * kTcBK;
+        if (s < nst) {
+          if constexpr (kMN) {
+            tc_load_mn<kTcBM>(sa + s * kTcSlabA, g.A, g.sak, ra, m0, ks, ke, tid);
+            tc_load_mn<kTcBN>(sbb + s * kTcSlabB, g.B, g.sbk, rb, n0, ks, ke, tid);
+          } else {
+            tc_load_kmajor<kTcBM>(sa + s * kTcSlabA, g.A, g.sam, g.M, m0, ks, ke, tid);
+            tc_load_kmajor<kTcBN>(sbb + s * kTcSlabB, g.B, g.sbn, g.N, n0, ks, ke, tid);
+          }
+        }
+        cp_async_commit();
       }
-      fence_async_smem();
     }
+#pragma unroll
+    for (int s = 0; s < kTcSlabs; ++s) {
+      if (s == 0) cp_async_wait<3>();
+      else if (s == 1) cp_async_wait<2>();
+      else if (s == 2) cp_async_wait<1>();
+      else cp_async_wait<0>();
+      fence_async_smem();
+      tc_fence_before();
+      __syncthreads();   // slab s (and, the first time, the tensor memory and the barrier) is ready
+      if (s >= nst) continue;
+      if (tid == 0) {
+        tc_fence_after();
+        const int nsub = (min(kTcBK, ke - k0 - s * kTcBK) + 15) / 16;
+        for (int sub = 0; sub < nsub; ++sub) {
+          const uint32_t pa = sa + s * kTcSlabA + (kMN ? 2048u : 32u) * (uint32_t)sub,
+                         pb = sbb + s * kTcSlabB + (kMN ? 2048u : 32u) * (uint32_t)sub;
+          umma_bf16(s_tmem, kMN ? umma_desc_mn_sw128(pa) : umma_desc_sw128(pa),
+                    kMN ? umma_desc_mn_sw128(pb) : umma_desc_sw128(pb), idesc, (round | s | sub) ? 1u : 0u);
+        }
+        if (s == nst - 1) umma_commit(bar);
+      }
+    }
+  }
+  if (round == 0) {
+    tc_fence_before();
     __syncthreads();
   }
-  // the last slab's commit completes after every MMA of the tile
-  if (nst > 0) {
-    const int last = nst - 1;
-    if (!bar_wait(bar0 + 8u * (uint32_t)(last & 1), (uint32_t)((last >> 1) & 1), kTcSpins)) ok = false;
-  }
+  tc_fence_after();
+  taddr = s_tmem;
+  if (round > 0 && !bar_wait(bar, (uint32_t)((round - 1) & 1), kTcSpins)) ok = false;
   tc_fence_after();
   if (!__all_sync(0xffffffffu, ok)) ok = false;
+  const int q = warp & 3, c0 = 32 * (warp >> 2);
   if (ok) {
-    float *blk = reinterpret_cast<float *>(sm) + warp * (32 * 33);
-    for (int c0 = 0; c0 < ncols; c0 += 32) {
+    if (c0 < ncols) {
+      float *blk = reinterpret_cast<float *>(sm) + warp * (32 * 33);
       float v[32];
-      if (nst > 0) {
-        tmem_ld32(taddr + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, v);
+      if (round > 0) {
+        tmem_ld32(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
       } else {
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = 0.f;
       }
-      __syncwarp();
+      if constexpr (std::is_same<Epi, EpiOutLoss>::value) {
+        // a lane holds a row: its few outputs straight from there
+        const int m = m0 + 32 * q + lane;
+        double part = m < g.M ? epi.row(m, v) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (lane == 0 && part != 0.0) atomicAdd(epi.loss, part);
+      } else {
 #pragma unroll
       for (int i = 0; i < 32; ++i) blk[lane * 33 + i] = v[i];   // row lane, column i
       __syncwarp();
@@ -1102,22 +1201,23 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const GemmArgs g, const Epi epi
             float ld[16];
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
-              const int m = m0 + 32 * warp + h + r;
+              const int m = m0 + 32 * q + h + r;
               ld[r] = m < g.M ? epi.load(m, n) : 0.f;
             }
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
-              const int m = m0 + 32 * warp + h + r;
+              const int m = m0 + 32 * q + h + r;
               if (m < g.M) epi.apply(m, n, blk[(h + r) * 33 + lane], ld[r]);
             }
           }
         } else {
 #pragma unroll 8
           for (int r = 0; r < 32; ++r) {
-            const int m = m0 + 32 * warp + r;
+            const int m = m0 + 32 * q + r;
             if (m < g.M) epi(m, n, blk[r * 33 + lane]);
           }
         }
+      }
       }
     }
   } else if (lane == 0) {
@@ -1125,14 +1225,54 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const GemmArgs g, const Epi epi
   }
   tc_fence_before();
   __syncthreads();
-  if (!ok && tid == 0 && nst > 0) {
-    // drain: every MMA this CTA issued has completed before its tensor
-    // memory is released (bounded as every wait)
-    const int last = nst - 1;
-    bar_wait(bar0 + 8u * (uint32_t)(last & 1), (uint32_t)((last >> 1) & 1), kTcSpins);
-  }
+  // drain: every MMA this CTA issued has completed before its tensor memory
+  // is released (bounded as every wait)
+  if (!ok && tid == 0 && round > 0) bar_wait(bar, (uint32_t)((round - 1) & 1), kTcSpins);
   __syncthreads();
   if (warp == 0) tmem_dealloc(taddr, kTcBN);
+}
+
+template <class Epi>
+__global__ void __launch_bounds__(kTcThreads, 2) k_gemm_tc(const GemmArgs g, const Epi epi, unsigned *err) {
+  pdl_trigger();
+  gemm_tile<false>(g, blockIdx.y * kTcBM, blockIdx.x * kTcBN, 0, g.K, epi, err);
+}
+
+// Every layer's weight gradient in one launch: tiles of all layers times
+// chunks of the batch, each CTA one tile of one chunk's partial sum.
+struct WgradArgs {
+  const __nv_bfloat16 *h[4], *dz[4];   // inputs and output gradients of layers 1-4
+  int n, kchunk;
+  MlpGradWs ws;
+};
+constexpr int kWgradTiles1 = kNh / kTcBN, kWgradTiles2 = (kNh / kTcBM) * (kNh / kTcBN), kWgradTiles4 = kNh / kTcBM;
+constexpr int kWgradTiles = kWgradTiles1 + 2 * kWgradTiles2 + kWgradTiles4;
+__global__ void __launch_bounds__(kTcThreads, 2) k_wgrad_tc(const WgradArgs a, unsigned *err) {
+  pdl_trigger();
+  int t = blockIdx.x % kWgradTiles, l = 0;
+  const int z = blockIdx.x / kWgradTiles;
+  if (t >= kWgradTiles1) {
+    t -= kWgradTiles1;
+    l = 1 + t / kWgradTiles2;
+    t -= (l - 1) * kWgradTiles2;
+  }
+  const int nt = l == 3 ? 1 : kNh / kTcBN;   // tiles along n
+  GemmArgs g;
+  g.A = l == 0 ? a.h[0] : l == 1 ? a.h[1] : l == 2 ? a.h[2] : a.h[3];
+  g.B = l == 0 ? a.dz[0] : l == 1 ? a.dz[1] : l == 2 ? a.dz[2] : a.dz[3];
+  g.sam = g.sbn = 1;
+  g.sak = l == 0 ? kNinPad : kNh;
+  g.sbk = l == 3 ? kNoutPad : kNh;
+  g.M = l == 0 ? kNin : kNh;
+  g.N = l == 3 ? kNout : kNh;
+  g.K = a.n;
+  g.kchunk = a.kchunk;
+  const long long len = (long long)g.M * g.N;
+  const long long off = l == 0 ? grad_ws_off(0) : l == 1 ? grad_ws_off(1) : l == 2 ? grad_ws_off(2) : grad_ws_off(3);
+  const int kb = z * a.kchunk;
+  gemm_tile<true>(g, t / nt * kTcBM, t % nt * kTcBN, kb, min(a.n, kb + a.kchunk),
+                  EpiStore{a.ws.ws + a.ws.nsplit * off + z * len, g.N}, err, l == 0 ? kNinPad : kNh,
+                  l == 3 ? kNoutPad : kNh);
 }
 
 }  // namespace casim_dev

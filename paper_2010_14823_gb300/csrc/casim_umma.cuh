@@ -35,11 +35,25 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
   return d;
 }
 
-// instruction descriptor, kind::f16: BF16 A and B (K-major), FP32 accumulator, M x N
-__host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
+// MN-major tiles with the 128-byte swizzle: a block of 64 rows (m or n) and 64
+// k is 64 k-rows of 128 contiguous bytes (eight 16-byte chunks of 8 rows
+// each), chunk j of k-row k at chunk position j ^ (k % 8); further blocks of
+// 64 rows follow 8192 bytes apart (the leading-dimension offset), groups of 8
+// k-rows 1024 bytes apart (the stride-dimension offset).
+__device__ __forceinline__ uint32_t sw128_mn_offset(int r, int k) {
+  return (uint32_t)((r >> 6) * 8192 + k * 128 + (((r >> 3) & 7) ^ (k & 7)) * 16);
+}
+__device__ __forceinline__ uint64_t umma_desc_mn_sw128(uint32_t saddr) {
+  return (umma_desc_sw128(saddr) & ~((uint64_t)0x3FFF << 16)) | (uint64_t)(8192u >> 4) << 16;
+}
+
+// instruction descriptor, kind::f16: BF16 A and B (K-major, or both MN-major),
+// FP32 accumulator, M x N
+__host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N, bool mn_major = false) {
   return (1u << 4)            // D format: F32
          | (1u << 7)          // A format: BF16
          | (1u << 10)         // B format: BF16
+         | (mn_major ? 3u << 15 : 0u)
          | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
@@ -62,6 +76,12 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, u
       "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+
+// Programmatic dependent launch: the next kernel of the stream may start its
+// prologue (pdl_trigger) and waits for this one's completion before it touches
+// memory (pdl_wait).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // all prior tcgen05 operations of this thread arrive on the mbarrier when done
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
