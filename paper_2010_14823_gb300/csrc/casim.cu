@@ -257,7 +257,13 @@ extern "C" int casim_init(casim_ctx **out, const casim_params *params, int preci
   if (e == cudaSuccess) e = StepWarm3::allow_smem();
   if (e == cudaSuccess) e = StepAero::allow_smem();
   if (e == cudaSuccess) e = Step3::allow_smem();
-  // and the batched step's (256-thread blocks: a 64 KB stage)
+  // and the batched step's (256-thread blocks: a 64 KB stage; the FP64 tile)
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_step_batch<PolicyF64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)batch_smem_bytes<PolicyF64>(kBatchNarrowBlock, kMaxLev));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_step_batch<PolicyF64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)batch_smem_bytes<PolicyF64>(kBatchMaxBlock, kMaxLev));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_step_batch<PolicyMix, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)batch_smem_bytes<PolicyMix>(kBatchNarrowBlock, kMaxLev));
@@ -1100,11 +1106,15 @@ extern "C" int casim_step_noalloc(const casim_params *params, int precision, con
   if (precision == CASIM_MIXED) {
     k_compact<PolicyMix><<<ntiles, kTile, 0, st>>>(a, sc->tiles, ntiles, kp);
     const size_t smem = batch_smem_bytes<PolicyMix>(kTile, nlev);
+    CUDA_TRY(cudaFuncSetAttribute(batch_kernel<PolicyMix>(kTile), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)batch_smem_bytes<PolicyMix>(kTile, kMaxLev)));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<PolicyMix>(kTile), kTile, smem));
     batch_kernel<PolicyMix>(kTile)<<<std::min(ntiles, std::max(1, per_sm) * nsm), kTile, smem, st>>>(a, kp);
   } else {
     k_compact<PolicyF64><<<ntiles, kTile, 0, st>>>(a, sc->tiles, ntiles, kp);
     const size_t smem = batch_smem_bytes<PolicyF64>(kTile, nlev);
+    CUDA_TRY(cudaFuncSetAttribute(batch_kernel<PolicyF64>(kTile), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)batch_smem_bytes<PolicyF64>(kTile, kMaxLev)));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<PolicyF64>(kTile), kTile, smem));
     batch_kernel<PolicyF64>(kTile)<<<std::min(ntiles, std::max(1, per_sm) * nsm), kTile, smem, st>>>(a, kp);
   }

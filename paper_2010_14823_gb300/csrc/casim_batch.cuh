@@ -55,8 +55,13 @@ struct BatchArgs {
 // dynamic shared memory of the batched step: the mixed step's prefetch stage
 // (two levels of 16 fields per thread) and the level tables of maxlev levels
 template <class M>
+__host__ __device__ constexpr size_t batch_stage_bytes(int block) {
+  if constexpr (M::kMixed) return stage_bytes<M>(block);
+  else return sizeof(F64Tile<M>);   // the FP64 sweep's tile
+}
+template <class M>
 __host__ __device__ constexpr size_t batch_smem_bytes(int block, int maxlev) {
-  return (step_staged<M, false>() ? stage_bytes<M>(block) : 0) + (size_t)maxlev * 24;
+  return batch_stage_bytes<M>(block) + (size_t)maxlev * 24;
 }
 
 template <class M>
@@ -124,9 +129,7 @@ __global__ void __launch_bounds__(kNarrow ? kBatchNarrowBlock : kBatchMaxBlock,
   extern __shared__ __align__(16) unsigned char batch_dyn[];
   __shared__ int s_item;
   const int B = blockDim.x;
-  constexpr bool kStage = step_staged<M, false>();
-  double *stage = kStage ? reinterpret_cast<double *>(batch_dyn) : nullptr;
-  double *s_dz = reinterpret_cast<double *>(batch_dyn + (kStage ? stage_bytes<M>(B) : 0));
+  double *s_dz = reinterpret_cast<double *>(batch_dyn + batch_stage_bytes<M>(B));
   double *s_dzdt = s_dz + b.maxlev;
   float *s_dtdz_f = reinterpret_cast<float *>(s_dzdt + b.maxlev), *s_dzdt_f = s_dtdz_f + b.maxlev;
   const LevelTab lt{s_dz, s_dzdt, s_dtdz_f, s_dzdt_f};
@@ -149,22 +152,22 @@ __global__ void __launch_bounds__(kNarrow ? kBatchNarrowBlock : kBatchMaxBlock,
     const int n = b.compact ? b.count[item.dom] : d.ncols;
     if (item.chunk * B < n) {
       const int idx = item.chunk * B + tid;
+      const int c = idx >= n ? -1 : b.compact && CASIM_INDEX_OK(idx < d.ncols, b.err) ? b.list[d.list_off + idx] : idx;
       KArgs a;
-      int c = 0;
-      if (idx < n) {
-        c = b.compact && CASIM_INDEX_OK(idx < d.ncols, b.err) ? b.list[d.list_off + idx] : idx;
-        a.fld = d.fld;
-        a.pitch = d.pitch;
-        a.dz = d.dz;
-        a.precip = d.precip;
-        a.err = b.err;
-        a.ncols = d.ncols;
-        a.nlev = d.nlev;
-        a.dt = b.dt;
-        a.surr = b.surr ? b.surr + d.pt_off : nullptr;
-        a.stats = nullptr;
-        a.segs = 1;
-        if (kStage) stage_level<M>(a, d.nlev - 1, c, stage + tid, B);   // in flight while the tables are made
+      a.fld = d.fld;
+      a.pitch = d.pitch;
+      a.dz = d.dz;
+      a.precip = d.precip;
+      a.err = b.err;
+      a.ncols = d.ncols;
+      a.nlev = d.nlev;
+      a.dt = b.dt;
+      a.surr = b.surr ? b.surr + d.pt_off : nullptr;
+      a.stats = nullptr;
+      a.segs = 1;
+      double *mine = reinterpret_cast<double *>(batch_dyn) + tid;   // the prefetch stage's slots (mixed)
+      if constexpr (M::kMixed) {
+        if (c >= 0) stage_level<M>(a, d.nlev - 1, c, mine, B);   // in flight while the tables are made
       }
       if (item.dom != prev_dom) {
         for (int k = tid; k < d.nlev; k += B) level_tab(s_dz, s_dzdt, s_dtdz_f, s_dzdt_f, k, d.dz[k], b.dt);
@@ -174,9 +177,19 @@ __global__ void __launch_bounds__(kNarrow ? kBatchNarrowBlock : kBatchMaxBlock,
       bool fast = true;
 #pragma unroll
       for (int x = 1; x < 5; ++x) fast &= one_substep(P.vmax[x], b.dt, d.dzmin, P.c_max);
-      if (idx < n)
-        eflag |= run_column<M, false, kStage, false, false, false>(a, P, lt, fast, c, Segment<false>(d.nlev), nullptr,
-                                                                   nullptr, kStage ? stage + tid : nullptr, B, nullptr);
+      if constexpr (M::kMixed) {
+        if (c >= 0)
+          eflag |= run_column<M, false, false, false, false>(a, P, lt, fast, c, Segment<false>(d.nlev), nullptr, nullptr,
+                                                             mine, B, nullptr);
+      } else {
+        // the FP64 sweep takes the item's columns 32 at a time
+        F64Tile<M> &t = *reinterpret_cast<F64Tile<M> *>(batch_dyn);
+        for (int w = 0; w < B / kF64Cols && item.chunk * B + w * kF64Cols < n; ++w) {
+          if (tid / kF64Cols == w) t.col[tid % kF64Cols] = c;
+          __syncthreads();
+          eflag |= f64_sweep<M, false>(a, P, lt, fast, Segment<true>(d.nlev, 0, 1, 1), nullptr, t);
+        }
+      }
     }
     // shared memory (item, dz) is reused by the next item; with one item per
     // block there is none, and the warps leave as they finish

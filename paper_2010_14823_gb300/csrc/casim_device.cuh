@@ -1585,14 +1585,10 @@ __device__ __forceinline__ void level_tab(double *dz, double *dzdt, float *dtdz_
   dzdt_f[k] = d2f(v / dt);
 }
 
-// The step kernel's dynamic shared memory: the prefetch stage (mixed step:
-// two levels of the fields the configuration loads, per thread), then the
-// level tables of this domain's nlev levels (dz, dz/dt, dt/dz and dz/dt in
-// FP32), then the block's reduction slots.
-template <class M, bool kTend>
-__host__ __device__ constexpr bool step_staged() {
-  return M::kMixed;
-}
+// The mixed step kernel's dynamic shared memory: the prefetch stage (two
+// levels of the fields the configuration loads, per thread), then the level
+// tables of this domain's nlev levels (dz, dz/dt, dt/dz and dz/dt in FP32),
+// then the block's reduction slots.
 // fields a configuration loads per point: the warm configuration T, qv, qc,
 // qr, nc, nr, na, p, rho, w; the cold one the 16 standard fields; then the
 // aerosol masses or sixth moments (fields 16..)
@@ -1609,34 +1605,30 @@ template <class M>
 __host__ __device__ constexpr size_t stage_bytes(int block) {
   return 2 * (size_t)stage_nf<M>() * block * sizeof(double);
 }
-// the split step's exchange slots, where the policy has no stage (one with a
-// stage uses the stage's, free by then): per thread one per sedimenting species
-__host__ __device__ constexpr size_t xch_bytes(int block) { return 4 * (size_t)block * sizeof(double); }
-template <class M, bool kTend, bool kSplit>
-__host__ __device__ constexpr size_t step_stage_bytes() {
-  return step_staged<M, kTend>() ? stage_bytes<M>(kBlock) : kSplit ? xch_bytes(kBlock) : 0;
-}
-template <class M, bool kTend, bool kSplit>
+template <class M>
 __host__ __device__ constexpr size_t step_smem_bytes(int nlev) {
-  return step_stage_bytes<M, kTend, kSplit>() + (size_t)nlev * 24 + (kBlock / 32) * 8;
+  return stage_bytes<M>(kBlock) + (size_t)nlev * 24 + (kBlock / 32) * 8;
 }
 
 struct StepSmem {
-  double *stage;   // [2][fields][kBlock], or the exchange slots [4][kBlock] of a policy without a stage
+  double *stage;   // [2][fields][kBlock] (staged policies)
   LevelTab lt;
   double *red;
 };
 
-template <class M, bool kTend, bool kSplit>
-__device__ __forceinline__ StepSmem step_smem(unsigned char *base, int nlev) {
+__device__ __forceinline__ StepSmem level_smem(unsigned char *p, int nlev) {
   StepSmem m;
-  unsigned char *p = base;
-  m.stage = reinterpret_cast<double *>(p);
-  p += step_stage_bytes<M, kTend, kSplit>();
+  m.stage = nullptr;
   double *dz = reinterpret_cast<double *>(p), *dzdt = dz + nlev;
   float *dtdz_f = reinterpret_cast<float *>(dzdt + nlev), *dzdt_f = dtdz_f + nlev;
   m.lt = LevelTab{dz, dzdt, dtdz_f, dzdt_f};
   m.red = reinterpret_cast<double *>(dzdt_f + nlev);   // 24 nlev bytes in: 8-byte aligned
+  return m;
+}
+template <class M>
+__device__ __forceinline__ StepSmem step_smem(unsigned char *base, int nlev) {
+  StepSmem m = level_smem(base + stage_bytes<M>(kBlock), nlev);
+  m.stage = reinterpret_cast<double *>(base);
   return m;
 }
 
@@ -1904,7 +1896,7 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
 // sweep of the processes (one read and one write of the state).  Otherwise
 // the processes are applied first and each species is sedimented with its
 // own substep count in further sweeps over the column.
-// stg (kStage): this thread's slots of the prefetch stage (slot f of buffer
+// The mixed form's sweep.  stg: this thread's slots of the prefetch stage (slot f of buffer
 // b at stg[(b * 16 + f) * ss], ss the block's thread count): level k - 1's 16
 // fields are copied there by cp.async while level k is processed, so the
 // sweep seldom waits on a load (each thread reads only the slots it filled
@@ -1927,23 +1919,22 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
 // keeps an owner from storing its lowest level before the thread below has
 // read it.  xch: this thread's exchange slots (stride ss), one per
 // sedimenting species.
-template <class M, bool fast, bool kTend, bool kStage, bool kStats, bool kLine, bool kSplit>
+template <class M, bool fast, bool kTend, bool kStats, bool kLine, bool kSplit>
 __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &P, const LevelTab &lt, int c,
                                                  const Segment<kSplit> &sg, double *xch, double *tend, double *stg,
                                                  int ss, ColStats *cs) {
-  static_assert(!kLine || (kStage && !kTend && !kStats), "whole-line stores re-read the stage");
-  const double *sdz = lt.dz, *sdzdt = lt.dzdt;
+  static_assert(M::kMixed, "the FP64 form has its own sweep");
+  static_assert(!kLine || (!kTend && !kStats), "whole-line stores: the in-place step");
+  const double *sdz = lt.dz;
   constexpr int kNf = stage_nf<M>();
   constexpr bool kShare = kSplit && fast && !kTend;   // the barrier above
   const int kfirst = fast ? sg.kfirst() : sg.ktop();
-  if constexpr (kStage) {
-    if (!CASIM_INDEX_OK(c >= 0 && c < a.ncols && c < a.pitch, a.err)) return 0u;
-    if constexpr (kSplit && !fast) {
-      // no flux is carried here: the first level is ktop, not the one the
-      // caller staged
-      cp_async_wait<0>();
-      stage_level<M>(a, kfirst, c, stg, ss);
-    }
+  if (!CASIM_INDEX_OK(c >= 0 && c < a.ncols && c < a.pitch, a.err)) return 0u;
+  if constexpr (kSplit && !fast) {
+    // no flux is carried here: the first level is ktop, not the one the caller
+    // staged
+    cp_async_wait<0>();
+    stage_level<M>(a, kfirst, c, stg, ss);
   }
   using R = typename M::R;
   using Ph = Phys<M>;
@@ -1964,203 +1955,137 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
     for (int i = 0; i < (a.nlev + 31) / 32; ++i) lvmask[i] = 0u;
   for (int k = kfirst; k >= sg.kbot(); --k) {
     Pt s;
-    const double *cur = nullptr;   // this level's slots of the stage (kStage)
-    if constexpr (kStage) {
-      const int b = (kfirst - k) & 1;
-      cur = stg + b * kNf * ss;
-      if (k > sg.kbot()) {
-        stage_level<M>(a, k - 1, c, stg + (b ^ 1) * kNf * ss, ss);
-        cp_async_wait<1>();   // this level's copies (the older group) have landed
-      } else {
-        cp_async_wait<0>();
-      }
-      if constexpr (!M::kWarm && !M::kAero && !M::kTri) {
-        s.T = cur[0 * ss]; s.qv = cur[1 * ss]; s.qc = cur[2 * ss]; s.qr = cur[3 * ss];
-        s.qi = cur[4 * ss]; s.qs = cur[5 * ss]; s.qg = cur[6 * ss];
-        s.nc = cur[7 * ss]; s.nr = cur[8 * ss]; s.ni = cur[9 * ss]; s.ns = cur[10 * ss];
-        s.ng = cur[11 * ss]; s.na = cur[12 * ss];
-        s.p = cur[13 * ss]; s.rho = cur[14 * ss]; s.w = cur[15 * ss];
-      } else {
-        if constexpr (M::kWarm) s.qi = s.qs = s.qg = s.ni = s.ns = s.ng = 0.0;
-#pragma unroll
-        for (int i = 0; i < kNf; ++i) pt_field<M>(s, stage_field<M>(i)) = cur[i * ss];
-      }
+    const int b = (kfirst - k) & 1;
+    const double *cur = stg + b * kNf * ss;   // this level's slots of the stage
+    if (k > sg.kbot()) {
+      stage_level<M>(a, k - 1, c, stg + (b ^ 1) * kNf * ss, ss);
+      cp_async_wait<1>();   // this level's copies (the older group) have landed
     } else {
-      load_pt<M::kWarm, M::kAero, M::kTri>(a, k, c, s);
+      cp_async_wait<0>();
+    }
+    if constexpr (!M::kWarm && !M::kAero && !M::kTri) {
+      s.T = cur[0 * ss]; s.qv = cur[1 * ss]; s.qc = cur[2 * ss]; s.qr = cur[3 * ss];
+      s.qi = cur[4 * ss]; s.qs = cur[5 * ss]; s.qg = cur[6 * ss];
+      s.nc = cur[7 * ss]; s.nr = cur[8 * ss]; s.ni = cur[9 * ss]; s.ns = cur[10 * ss];
+      s.ng = cur[11 * ss]; s.na = cur[12 * ss];
+      s.p = cur[13 * ss]; s.rho = cur[14 * ss]; s.w = cur[15 * ss];
+    } else {
+      if constexpr (M::kWarm) s.qi = s.qs = s.qg = s.ni = s.ns = s.ng = 0.0;
+#pragma unroll
+      for (int i = 0; i < kNf; ++i) pt_field<M>(s, stage_field<M>(i)) = cur[i * ss];
     }
     if constexpr (kShare) {
       if (k == kfirst) split_arrive();   // the level above the segment has been read
     }
-    bool touched;
-    if constexpr (!M::kMixed) {
-      eflag |= nonfinite_in(s);
-      // the aerosol masses or sixth moments too: an inactive point is not stored,
-      // so its values are checked as they are read
+    W<float> w;
+    float es0, qs0;
+    const bool act = MixT<M>::active(K, s, P.T0, w, es0, qs0);
+    // the aerosol masses or sixth moments join the magnitude scan (an
+    // inactive point is not stored, so its values are checked as read)
 #pragma unroll
-      for (int e = 0; e < nextra<M>(); ++e) eflag |= nonfinite(extra<M>(s, e));
-      double es0, qs0;
-      touched = F64T<M>::active(K, s, es0, qs0);
-      if constexpr (kStats) cs->active += touched;
-      double mu3[4];
-      unsigned keep3 = 0;   // species whose shape the processes left unchanged (triple-moment policies)
-      if (touched) F64T<M>::process(K, s, a.dt, es0, qs0, mu3, &keep3);
-      if constexpr (fast) {
-        const double dzk = sdz[k];
-        const double dfac = ::exp(0.4 * (K.lgrho0 - ::log(s.rho)));
+    for (int e = 0; e < nextra<M>(); ++e) w.hmax = max(w.hmax, hiabs(extra<M>(s, e)));
+    if constexpr (kStats) cs->active += act;
+    MixInc o;
+    MassAcc macc;
+    unsigned keep3 = 0;   // species whose shape the processes left unchanged (triple-moment policies)
+    float dn[4] = {0.f, 0.f, 0.f, 0.f};   // number increments of r, i, s, g
+    float qpost[4], npost[4];
+    if (act) {
+      MixT<M>::template process<kTend>(K, s, a.dt, w, es0, qs0, o, a.surr ? a.surr + (size_t)k * a.pitch + c : nullptr);
+      if constexpr (!M::kWarm && !M::kAero && !M::kTri) {
+        // the FP64 values the increments are added to, read again from this
+        // level's stage slots (they stay there until the level after next is
+        // prefetched) rather than held in registers through the processes:
+        // no spills, 2.02 -> 1.95 ms per 512x512x150 step, results unchanged
+        const volatile double *v = cur;
+        s.T = v[0 * ss]; s.qv = v[1 * ss]; s.qc = v[2 * ss]; s.qr = v[3 * ss];
+        s.qi = v[4 * ss]; s.qs = v[5 * ss]; s.qg = v[6 * ss];
+        s.nc = v[7 * ss]; s.nr = v[8 * ss]; s.ni = v[9 * ss]; s.ns = v[10 * ss];
+        s.ng = v[11 * ss]; s.na = v[12 * ss]; s.rho = v[14 * ss];
+      }
+      MixT<M>::apply_masses(s, o, macc);
+      if constexpr (M::kTri) keep3 = MixT<M>::apply_z(K, s, w, o);
+      if (o.dn[0] != 0.f) s.nc += f2d(o.dn[0]);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) dn[x] = o.dn[1 + x];
+      // post-process FP32 masses and numbers for the fall speeds
+      qpost[0] = w.qr + o.cr - o.rv + o.xr[0] + o.xr[1] + o.xr[2];
+      qpost[1] = w.qx[0] + o.vx[0] - o.xr[0];
+      qpost[2] = w.qx[1] + o.vx[1] - o.xr[1];
+      qpost[3] = w.qx[2] + o.vx[2] + o.cg - o.xr[2];
+      npost[0] = w.nr + dn[0];
+#pragma unroll
+      for (int x = 1; x < 4; ++x) npost[x] = w.nx[x - 1] + dn[x];
+    } else {
+      qpost[0] = w.qr;
+      qpost[1] = w.qx[0];
+      qpost[2] = w.qx[1];
+      qpost[3] = w.qx[2];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) npost[x] = 0.f;   // read only where a species is present
+    }
+    bool touched = act;
+    if constexpr (fast) {
+      bool any = false;
+#pragma unroll
+      for (int x = 0; x < kSed; ++x) any |= qpost[x] > K.qmin || Fq[x] != 0.f || Fn[x] != 0.f;
+      if (any) {
+        if (!act) w.hmax = max(w.hmax, hiabs(s.rho));
+        const float rho = act ? w.rho : d2f(s.rho);
+        const float dfac = ex2a(0.4f * (K.lgrho0 - lg2a(rho)));
+        const float sc = __fdividef(lt.dtdz_f[k], d2f_rn(s.rho));
+        const float guard = lt.dzdt_f[k];
 #pragma unroll
         for (int x = 0; x < kSed; ++x) {
-          double &q = qref(s, x);
-          double &n = nref(s, x);
-          double F = 0, G = 0, A = 0, H = 0;
-          if (q > K.qmin) {
-            double vq, vn;
+          float F = 0.f, G = 0.f, A = 0.f, H = 0.f;
+          if (qpost[x] > K.qmin) {
+            const float n = act ? npost[x] : d2f(nref(s, x));
+            float vq, vn;
             if (x < nz3<M>()) {
-              double vz;
-              const double z = zref(s, x);
-              const double mus = ((keep3 >> x) & 1u) ? mu3[x] : Shape3<M>::mu(K, x, q, n, z);
-              Shape3<M>::fall_speeds_mu(K, x, sdzdt[k], ::log(q), n, mus, dfac, vq, vn, vz);
-              H = s.rho * (z > 0.0 ? z : 0.0) * vz;
+              float vz;
+              const float zp = d2f(zref(s, x));
+              const float mus = ((keep3 >> x) & 1u) ? w.mu3[x] : Shape3<M>::mu(K, x, qpost[x], n, zp);
+              Shape3<M>::fall_speeds_mu(K, x, guard, lg2a(qpost[x]), n, mus, dfac, vq, vn, vz);
+              H = rho * fmaxf(zp, 0.f) * vz;
             } else {
-              Ph::fall_speeds(K, sdzdt[k], ::log(q), n, dfac, x, vq, vn);
+              Ph::fall_speeds(K, guard, lg2a(qpost[x]), n, dfac, x, vq, vn);
             }
-            F = s.rho * q * vq;
-            G = s.rho * (n > 0.0 ? n : 0.0) * vn;
-            if (x < na3<M>()) A = s.rho * maref(s, x) * vq;
+            F = rho * qpost[x] * vq;
+            G = rho * fmaxf(n, 0.f) * vn;
+            if (x < na3<M>()) A = rho * d2f(maref(s, x)) * vq;
           }
           if (x < nz3<M>()) {
-            if (H != 0.0 || Fz[x] != 0.0) {
-              zref(s, x) += a.dt * (Fz[x] - H) / (s.rho * dzk);
+            if (H != 0.f || Fz[x] != 0.f) {
+              zref(s, x) += f2d((Fz[x] - H) * sc);
               touched = true;
             }
             Fz[x] = H;
           }
-          if (F != 0.0 || Fq[x] != 0.0 || G != 0.0 || Fn[x] != 0.0) {
-            q += a.dt * (Fq[x] - F) / (s.rho * dzk);
-            n += a.dt * (Fn[x] - G) / (s.rho * dzk);
-            touched = true;
-          }
           if (x < na3<M>()) {
-            if (A != 0.0 || Fa[x] != 0.0) {
-              maref(s, x) += a.dt * (Fa[x] - A) / (s.rho * dzk);
+            if (A != 0.f || Fa[x] != 0.f) {
+              maref(s, x) += f2d((Fa[x] - A) * sc);
               touched = true;
             }
             Fa[x] = A;
+          }
+          if (F != 0.f || Fq[x] != 0.f) {
+            macc.add(x == 0 ? MassAcc::kR : MassAcc::kI + x - 1, (Fq[x] - F) * sc);
+            touched = true;
+          }
+          if (G != 0.f || Fn[x] != 0.f) {
+            dn[x] += (Fn[x] - G) * sc;
+            touched = true;
           }
           Fq[x] = F;
           Fn[x] = G;
         }
       }
-    } else {
-      W<float> w;
-      float es0, qs0;
-      const bool act = MixT<M>::active(K, s, P.T0, w, es0, qs0);
-      // the aerosol masses or sixth moments join the magnitude scan (an
-      // inactive point is not stored, so its values are checked as read)
-#pragma unroll
-      for (int e = 0; e < nextra<M>(); ++e) w.hmax = max(w.hmax, hiabs(extra<M>(s, e)));
-      if constexpr (kStats) cs->active += act;
-      MixInc o;
-      MassAcc macc;
-      unsigned keep3 = 0;   // species whose shape the processes left unchanged (triple-moment policies)
-      float dn[4] = {0.f, 0.f, 0.f, 0.f};   // number increments of r, i, s, g
-      float qpost[4], npost[4];
-      if (act) {
-        MixT<M>::template process<kTend>(K, s, a.dt, w, es0, qs0, o, a.surr ? a.surr + (size_t)k * a.pitch + c : nullptr);
-        if constexpr (kStage && !M::kWarm && !M::kAero && !M::kTri) {
-          // the FP64 values the increments are added to, read again from this
-          // level's stage slots (they stay there until the level after next is
-          // prefetched) rather than held in registers through the processes:
-          // no spills, 2.02 -> 1.95 ms per 512x512x150 step, results unchanged
-          const volatile double *v = cur;
-          s.T = v[0 * ss]; s.qv = v[1 * ss]; s.qc = v[2 * ss]; s.qr = v[3 * ss];
-          s.qi = v[4 * ss]; s.qs = v[5 * ss]; s.qg = v[6 * ss];
-          s.nc = v[7 * ss]; s.nr = v[8 * ss]; s.ni = v[9 * ss]; s.ns = v[10 * ss];
-          s.ng = v[11 * ss]; s.na = v[12 * ss]; s.rho = v[14 * ss];
-        }
-        MixT<M>::apply_masses(s, o, macc);
-        if constexpr (M::kTri) keep3 = MixT<M>::apply_z(K, s, w, o);
-        if (o.dn[0] != 0.f) s.nc += f2d(o.dn[0]);
-#pragma unroll
-        for (int x = 0; x < 4; ++x) dn[x] = o.dn[1 + x];
-        // post-process FP32 masses and numbers for the fall speeds
-        qpost[0] = w.qr + o.cr - o.rv + o.xr[0] + o.xr[1] + o.xr[2];
-        qpost[1] = w.qx[0] + o.vx[0] - o.xr[0];
-        qpost[2] = w.qx[1] + o.vx[1] - o.xr[1];
-        qpost[3] = w.qx[2] + o.vx[2] + o.cg - o.xr[2];
-        npost[0] = w.nr + dn[0];
-#pragma unroll
-        for (int x = 1; x < 4; ++x) npost[x] = w.nx[x - 1] + dn[x];
-      } else {
-        qpost[0] = w.qr;
-        qpost[1] = w.qx[0];
-        qpost[2] = w.qx[1];
-        qpost[3] = w.qx[2];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) npost[x] = 0.f;   // read only where a species is present
-      }
-      touched = act;
-      if constexpr (fast) {
-        bool any = false;
-#pragma unroll
-        for (int x = 0; x < kSed; ++x) any |= qpost[x] > K.qmin || Fq[x] != 0.f || Fn[x] != 0.f;
-        if (any) {
-          if (!act) w.hmax = max(w.hmax, hiabs(s.rho));
-          const float rho = act ? w.rho : d2f(s.rho);
-          const float dfac = ex2a(0.4f * (K.lgrho0 - lg2a(rho)));
-          const float sc = __fdividef(lt.dtdz_f[k], d2f_rn(s.rho));
-          const float guard = lt.dzdt_f[k];
-#pragma unroll
-          for (int x = 0; x < kSed; ++x) {
-            float F = 0.f, G = 0.f, A = 0.f, H = 0.f;
-            if (qpost[x] > K.qmin) {
-              const float n = act ? npost[x] : d2f(nref(s, x));
-              float vq, vn;
-              if (x < nz3<M>()) {
-                float vz;
-                const float zp = d2f(zref(s, x));
-                const float mus = ((keep3 >> x) & 1u) ? w.mu3[x] : Shape3<M>::mu(K, x, qpost[x], n, zp);
-                Shape3<M>::fall_speeds_mu(K, x, guard, lg2a(qpost[x]), n, mus, dfac, vq, vn, vz);
-                H = rho * fmaxf(zp, 0.f) * vz;
-              } else {
-                Ph::fall_speeds(K, guard, lg2a(qpost[x]), n, dfac, x, vq, vn);
-              }
-              F = rho * qpost[x] * vq;
-              G = rho * fmaxf(n, 0.f) * vn;
-              if (x < na3<M>()) A = rho * d2f(maref(s, x)) * vq;
-            }
-            if (x < nz3<M>()) {
-              if (H != 0.f || Fz[x] != 0.f) {
-                zref(s, x) += f2d((Fz[x] - H) * sc);
-                touched = true;
-              }
-              Fz[x] = H;
-            }
-            if (x < na3<M>()) {
-              if (A != 0.f || Fa[x] != 0.f) {
-                maref(s, x) += f2d((Fa[x] - A) * sc);
-                touched = true;
-              }
-              Fa[x] = A;
-            }
-            if (F != 0.f || Fq[x] != 0.f) {
-              macc.add(x == 0 ? MassAcc::kR : MassAcc::kI + x - 1, (Fq[x] - F) * sc);
-              touched = true;
-            }
-            if (G != 0.f || Fn[x] != 0.f) {
-              dn[x] += (Fn[x] - G) * sc;
-              touched = true;
-            }
-            Fq[x] = F;
-            Fn[x] = G;
-          }
-        }
-      }
-#pragma unroll
-      for (int x = 0; x < kSed; ++x)
-        if (dn[x] != 0.f) nref(s, x) += f2d(dn[x]);
-      macc.apply<M::kWarm>(s);
-      eflag |= w.hmax >= kF32RangeHi;
     }
+#pragma unroll
+    for (int x = 0; x < kSed; ++x)
+      if (dn[x] != 0.f) nref(s, x) += f2d(dn[x]);
+    macc.apply<M::kWarm>(s);
+    eflag |= w.hmax >= kF32RangeHi;
     if constexpr (!fast) courant<M>(a, K, sdz, k, s, Fq);   // the flux registers hold the Courant numbers
     if constexpr (kSplit && fast) {
       if (k > sg.ktop()) continue;   // the level above the segment: its flux only
@@ -2169,7 +2094,7 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
       }
     }
     if constexpr (kTend) {
-      eflag |= store_tend<M>(a, tend, k, c, s, fast, per_dt, kStage ? cur : nullptr, ss);
+      eflag |= store_tend<M>(a, tend, k, c, s, fast, per_dt, cur, ss);
     } else if constexpr (kLine) {
       const unsigned wm = __activemask();
       if (__any_sync(wm, touched)) {
@@ -2292,13 +2217,13 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
   return eflag;
 }
 
-// (kStage: the caller has staged level sg.kfirst() with stage_level)
-template <class M, bool kTend, bool kStage, bool kStats, bool kLine, bool kSplit>
+// (the caller has staged level sg.kfirst() with stage_level)
+template <class M, bool kTend, bool kStats, bool kLine, bool kSplit>
 __device__ __forceinline__ unsigned run_column(const KArgs &a, const KParams &P, const LevelTab &lt, bool fast, int c,
                                                const Segment<kSplit> &sg, double *xch, double *tend, double *stg,
                                                int ss, ColStats *cs) {
-  return fast ? sweep_column<M, true, kTend, kStage, kStats, kLine, kSplit>(a, P, lt, c, sg, xch, tend, stg, ss, cs)
-              : sweep_column<M, false, kTend, kStage, kStats, kLine, kSplit>(a, P, lt, c, sg, xch, tend, stg, ss, cs);
+  return fast ? sweep_column<M, true, kTend, kStats, kLine, kSplit>(a, P, lt, c, sg, xch, tend, stg, ss, cs)
+              : sweep_column<M, false, kTend, kStats, kLine, kSplit>(a, P, lt, c, sg, xch, tend, stg, ss, cs);
 }
 
 // one column's statistics into the buffer: warp sums, one atomic per warp
@@ -2322,8 +2247,21 @@ __device__ __forceinline__ void stats_add(unsigned long long *st, const ColStats
   }
 }
 
+}  // namespace casim_dev
+
+#include "casim_f64.cuh"
+
+namespace casim_dev {
+
+// Dynamic shared memory of the FP64 sweep: the tile, then (statistics build)
+// the counters, then the level tables and the block's reduction slots.
+template <class M, bool kStats = false>
+__host__ __device__ constexpr size_t f64_smem_bytes(int nlev) {
+  return sizeof(F64Tile<M>) + (kStats ? sizeof(F64Stats) : 0) + (size_t)nlev * 24 + 8 * 8;
+}
+
 // kTend: tendency mode (tend receives the source terms, a.fld unchanged).
-// Dynamic shared memory: step_smem_bytes<M, kTend, kSplit>(a.nlev).  kStats: the
+// Dynamic shared memory: step_smem_bytes<M>(a.nlev), FP64 f64_smem_bytes<M, kStats>(a.nlev).  kStats: the
 // statistics instantiation (standard configuration; a.stats set).  kLine:
 // whole-line stores for a state in mapped host memory (staged policies).
 //
@@ -2336,30 +2274,43 @@ __device__ __forceinline__ void stats_add(unsigned long long *st, const ColStats
 template <class M, bool kTend, bool kStats = false, bool kLine = false, bool kSplit = false>
 __global__ void __launch_bounds__(kBlock, M::kMinBlocks) k_step(const KArgs a, const KParams P, double *tend) {
   extern __shared__ __align__(16) unsigned char step_dyn[];
-  constexpr bool kStage = step_staged<M, kTend>();
-  const StepSmem sm = step_smem<M, kTend, kSplit>(step_dyn, a.nlev);
   ColStats cs{0, 0, {1, 1, 1, 1}};
-  double *mine = sm.stage + threadIdx.x;
   unsigned eflag;
-  if constexpr (kSplit) {
+  if constexpr (!M::kMixed) {
+    // the FP64 form: 32 columns per block, gridDim.y segments
+    F64Tile<M> &t = *reinterpret_cast<F64Tile<M> *>(step_dyn);
+    F64Stats *st = kStats ? reinterpret_cast<F64Stats *>(step_dyn + sizeof(F64Tile<M>)) : nullptr;
+    const StepSmem sm = level_smem(step_dyn + sizeof(F64Tile<M>) + (kStats ? sizeof(F64Stats) : 0), a.nlev);
+    const Segment<true> sg(a.nlev, blockIdx.y, gridDim.y, 1);
+    const bool fast = prologue<true>(a, P, sm, sg.kbot(), sg.kfirst());
+    if (threadIdx.x < kF64Cols) {
+      const int c = blockIdx.x * kF64Cols + threadIdx.x;
+      t.col[threadIdx.x] = c < a.ncols ? c : -1;
+    }
+    __syncthreads();
+    eflag = f64_sweep<M, kTend, kStats>(a, P, sm.lt, fast, sg, tend, t, st);
+  } else if constexpr (kSplit) {
+    const StepSmem sm = step_smem<M>(step_dyn, a.nlev);
+    double *mine = sm.stage + threadIdx.x;
     const int cols = kBlock / a.segs, nseg = gridDim.y * a.segs;
     const int c = blockIdx.x * cols + (int)(threadIdx.x & (cols - 1));
     const Segment<true> sg(a.nlev, blockIdx.y * a.segs + threadIdx.x / cols, nseg, a.segs);
     const Segment<true> s0(a.nlev, blockIdx.y * a.segs, nseg, a.segs), s1(a.nlev, (blockIdx.y + 1) * a.segs - 1, nseg, a.segs);
-    if (kStage && c < a.ncols) stage_level<M>(a, sg.kfirst(), c, mine, kBlock);
+    if (c < a.ncols) stage_level<M>(a, sg.kfirst(), c, mine, kBlock);
     const bool fast = prologue<true>(a, P, sm, s1.kbot(), s0.kfirst());
     if (c >= a.ncols) return;
-    eflag = run_column<M, kTend, kStage, kStats, kLine, true>(a, P, sm.lt, fast, c, sg, mine, tend,
-                                                              kStage ? mine : nullptr, kBlock, &cs);
+    eflag = run_column<M, kTend, kStats, kLine, true>(a, P, sm.lt, fast, c, sg, mine, tend, mine, kBlock, &cs);
   } else {
+    const StepSmem sm = step_smem<M>(step_dyn, a.nlev);
+    double *mine = sm.stage + threadIdx.x;
     const int c = blockIdx.x * kBlock + threadIdx.x;
-    if (kStage && c < a.ncols) stage_level<M>(a, a.nlev - 1, c, mine, kBlock);
+    if (c < a.ncols) stage_level<M>(a, a.nlev - 1, c, mine, kBlock);
     const bool fast = prologue<false>(a, P, sm, 0, 0);
     if (c >= a.ncols) return;
-    eflag = run_column<M, kTend, kStage, kStats, kLine, false>(a, P, sm.lt, fast, c, Segment<false>(a.nlev), nullptr, tend,
-                                                               kStage ? mine : nullptr, kBlock, &cs);
+    eflag = run_column<M, kTend, kStats, kLine, false>(a, P, sm.lt, fast, c, Segment<false>(a.nlev), nullptr, tend, mine,
+                                                       kBlock, &cs);
   }
-  if constexpr (kStats) stats_add(a.stats, cs);
+  if constexpr (kStats && M::kMixed) stats_add(a.stats, cs);
   if (eflag) atomicOr(a.err, eflag);
 }
 

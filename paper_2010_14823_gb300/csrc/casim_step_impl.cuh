@@ -26,6 +26,15 @@ inline int step_segments(int ncols, int nlev, int nsm, int blocks_per_sm, bool l
   return n;
 }
 
+// The FP64 sweep's segments per column group (1 to 8 blocks of a cluster): as
+// many as still fit in one resident wave, at least 4 levels each.
+inline int f64_segments(unsigned groups, int nlev, int nsm, int blocks_per_sm) {
+  const unsigned room = (unsigned)(nsm * blocks_per_sm);
+  int n = 1;
+  while (n < 8 && 8 * n <= nlev && 2 * n * groups <= room) n *= 2;
+  return n;
+}
+
 // grid.x column groups; the levels of a column shared by clusters of grid.y blocks
 template <class K>
 cudaError_t step_launch(K kernel, dim3 grid, size_t smem, cudaStream_t st, const KArgs &a, const KParams &kp,
@@ -45,28 +54,25 @@ cudaError_t step_launch(K kernel, dim3 grid, size_t smem, cudaStream_t st, const
   return cudaLaunchKernelEx(&cfg, kernel, a, kp, tend);
 }
 
-template <class M>
-cudaError_t step_allow_smem() {
+template <class PMix, class PF64>
+cudaError_t StepKernels<PMix, PF64>::allow_smem() {
   cudaError_t e = cudaSuccess;
   auto allow = [&](auto *kernel, size_t bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  allow(k_step<M, false>, step_smem_bytes<M, false, false>(kMaxLev));
-  allow(k_step<M, true>, step_smem_bytes<M, true, false>(kMaxLev));
-  allow(k_step<M, false, false, true>, step_smem_bytes<M, false, false>(kMaxLev));
-  allow(k_step<M, false, false, false, true>, step_smem_bytes<M, false, true>(kMaxLev));
-  allow(k_step<M, true, false, false, true>, step_smem_bytes<M, true, true>(kMaxLev));
-  allow(k_step<M, false, false, true, true>, step_smem_bytes<M, false, true>(kMaxLev));
-  return e;
-}
-
-template <class PMix, class PF64>
-cudaError_t StepKernels<PMix, PF64>::allow_smem() {
-  cudaError_t e = step_allow_smem<PMix>();
-  if constexpr (std::is_same<PMix, PolicyMix>::value)
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_step<PMix, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)step_smem_bytes<PMix, false, false>(kMaxLev));
+  const size_t mixed = step_smem_bytes<PMix>(kMaxLev), fp64 = f64_smem_bytes<PF64>(kMaxLev);
+  allow(k_step<PMix, false>, mixed);
+  allow(k_step<PMix, true>, mixed);
+  allow(k_step<PMix, false, false, true>, mixed);
+  allow(k_step<PMix, false, false, false, true>, mixed);
+  allow(k_step<PMix, true, false, false, true>, mixed);
+  allow(k_step<PMix, false, false, true, true>, mixed);
+  allow(k_step<PF64, false>, fp64);
+  allow(k_step<PF64, true>, fp64);
+  if constexpr (std::is_same<PMix, PolicyMix>::value) {
+    allow(k_step<PMix, false, true>, mixed);
+    allow(k_step<PF64, false, true>, f64_smem_bytes<PF64, true>(kMaxLev));
+  }
   return e;
 }
 
@@ -74,34 +80,35 @@ template <class PMix, class PF64>
 cudaError_t StepKernels<PMix, PF64>::launch(const StepLaunch &l, const KArgs &args, const KParams &kp) {
   KArgs a = args;
   const bool line = l.line && l.mixed;
+  const unsigned groups = (unsigned)((a.ncols + kF64Cols - 1) / kF64Cols);   // FP64 blocks
   const dim3 whole((unsigned)((a.ncols + kBlock - 1) / kBlock));
   if constexpr (std::is_same<PMix, PolicyMix>::value) {
     // the statistics build (a CASIM_STATS context: standard configuration)
     if (a.stats && !l.tend)
-      return l.mixed ? step_launch(k_step<PMix, false, true>, whole, step_smem_bytes<PMix, false, false>(a.nlev),
-                                   l.stream, a, kp, nullptr)
-                     : step_launch(k_step<PF64, false, true>, whole, step_smem_bytes<PF64, false, false>(a.nlev),
-                                   l.stream, a, kp, nullptr);
+      return l.mixed ? step_launch(k_step<PMix, false, true>, whole, step_smem_bytes<PMix>(a.nlev), l.stream, a, kp,
+                                   nullptr)
+                     : step_launch(k_step<PF64, false, true>, dim3(groups), f64_smem_bytes<PF64, true>(a.nlev), l.stream,
+                                   a, kp, nullptr);
   }
-  const int n = step_segments(a.ncols, a.nlev, l.nsm, l.mixed ? PMix::kMinBlocks : PF64::kMinBlocks, line);
-  auto go = [&](auto *one, auto *split, size_t smem1, size_t smem) {
-    if (n == 1) return step_launch(one, whole, smem1, l.stream, a, kp, l.tend);
+  if (!l.mixed) {
+    // FP64: blocks of 32 columns, a cluster of segments where they are few
+    const dim3 grid(groups, (unsigned)f64_segments(groups, a.nlev, l.nsm, PF64::kMinBlocks));
+    const size_t smem = f64_smem_bytes<PF64>(a.nlev);
+    return l.tend ? step_launch(k_step<PF64, true>, grid, smem, l.stream, a, kp, l.tend)
+                  : step_launch(k_step<PF64, false>, grid, smem, l.stream, a, kp, nullptr);
+  }
+  const int n = step_segments(a.ncols, a.nlev, l.nsm, PMix::kMinBlocks, line);
+  const size_t smem = step_smem_bytes<PMix>(a.nlev);
+  auto go = [&](auto *one, auto *split) {
+    if (n == 1) return step_launch(one, whole, smem, l.stream, a, kp, l.tend);
     a.segs = n < kBlock / 32 ? n : kBlock / 32;   // a warp per segment in the block, the rest over a cluster
     const int cols = kBlock / a.segs;
     return step_launch(split, dim3((unsigned)((a.ncols + cols - 1) / cols), (unsigned)(n / a.segs)), smem, l.stream, a,
                        kp, l.tend);
   };
-#define CASIM_STEP_PAIR(M, tend, line)                                                                \
-  go(k_step<M, tend, false, line>, k_step<M, tend, false, line, true>, step_smem_bytes<M, tend, false>(a.nlev), \
-     step_smem_bytes<M, tend, true>(a.nlev))
-  if (l.mixed) {
-    if (l.tend) return CASIM_STEP_PAIR(PMix, true, false);
-    if (line) return CASIM_STEP_PAIR(PMix, false, true);
-    return CASIM_STEP_PAIR(PMix, false, false);
-  }
-  if (l.tend) return CASIM_STEP_PAIR(PF64, true, false);
-  return CASIM_STEP_PAIR(PF64, false, false);
-#undef CASIM_STEP_PAIR
+  if (l.tend) return go(k_step<PMix, true>, k_step<PMix, true, false, false, true>);
+  if (line) return go(k_step<PMix, false, false, true>, k_step<PMix, false, false, true, true>);
+  return go(k_step<PMix, false>, k_step<PMix, false, false, false, true>);
 }
 
 }  // namespace casim_dev
