@@ -22,6 +22,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "casim_math64.cuh"
+
 namespace casim_dev {
 
 constexpr int kMaxLev = 1024;    // levels per column held in shared memory (dz)
@@ -65,6 +67,8 @@ struct ConstK {
   R mey_a, mey_b, mey_c, mi0;
   // air
   R mu_air, inv_dv, lgrho0, twopi;
+  R v0_ln;                          // FP64: ln of (mu_air/Dv)^(1/3) (rho0^0.4/mu_air)^(1/2)
+  R ls_cp, lf_cp;                   // Ls/cp, Lf/cp
   SpeciesK<R> sp[5];
   // triple-moment species r, i, s, g (index 0..3, species 1..4): what their
   // shape-dependent constants are built from
@@ -216,16 +220,16 @@ struct PolicyF64 {
   static __device__ __forceinline__ R toR(double x) { return x; }
   static __device__ __forceinline__ R toRn(double x) { return x; }
   static __device__ __forceinline__ double toD(R x) { return x; }
-  static __device__ __forceinline__ R exp(R x) { return ::exp(x); }
-  static __device__ __forceinline__ R lg(R x) { return ::log(x); }   // log in the constants' base
-  static __device__ __forceinline__ R ex(R x) { return ::exp(x); }   // inverse of lg
-  static __device__ __forceinline__ R ln(R x) { return ::log(x); }
+  static __device__ __forceinline__ R exp(R x) { return exp64(x); }
+  static __device__ __forceinline__ R lg(R x) { return log64(x); }   // log in the constants' base
+  static __device__ __forceinline__ R ex(R x) { return exp64(x); }   // inverse of lg
+  static __device__ __forceinline__ R ln(R x) { return log64(x); }
   static __device__ __forceinline__ R sqrt(R x) { return ::sqrt(x); }
   static __device__ __forceinline__ R cbrt(R x) { return ::cbrt(x); }
   static __device__ __forceinline__ R erfc(R x) { return ::erfc(x); }
   // Gamma(x + s) / Gamma(x)
   static __device__ __forceinline__ R gratio(R x, R s) { return ::exp(::lgamma(x + s) - ::lgamma(x)); }
-  static __device__ __forceinline__ R div(R a, R b) { return a / b; }
+  static __device__ __forceinline__ R div(R a, R b) { return div64(a, b); }
   static __device__ __forceinline__ R mn(R a, R b) { return a < b ? a : b; }
   static __device__ __forceinline__ R mx(R a, R b) { return a > b ? a : b; }
 };
@@ -363,6 +367,7 @@ __device__ __forceinline__ unsigned hiabs(double x) { return (unsigned)__double2
 // raw process rates (kg/kg/s; number rates for scc, scr, nucn)
 template <class R>
 struct Rt {
+  R dfac;   // (rho0/rho)^0.4 (FP64 form; zero where no species needs it)
   R aut, acc, scc, scr, evr, nucn, dep[3], rim[2], mlt[3];
 };
 
@@ -490,7 +495,7 @@ struct Phys {
   // from tc = T - T0 (formed in FP64) rather than from T rounded to FP32
   static __device__ __forceinline__ R es_ice(const ConstK<R> &K, double T, R tc) {
     if constexpr (!M::kMixed) {
-      return K.esi0 * ::exp(K.esia * (T - K.esit) / (T - K.esib));
+      return K.esi0 * exp64(div64(K.esia * (T - K.esit), T - K.esib));
     } else {
       return K.esi0 * M::exp(M::div(K.esia * (tc + K.t0_esit), tc + K.t0_esib));
     }
@@ -526,6 +531,17 @@ struct Phys {
     return M::mn(l, X.lghi);
   }
 
+  // the same from (q, n): the FP64 form takes one logarithm, of n/q
+  static __device__ __forceinline__ R lglam_q(const SpeciesK<R> &X, R q, R n) {
+    if constexpr (M::kMixed) {
+      return lglam(X, M::lg(q), n);
+    } else {
+      R l = (X.lglamfac + M::lg(M::div(M::mx(n, (R)0), q))) * X.invb;
+      l = M::mx(l, X.lglo);
+      return M::mn(l, X.lghi);
+    }
+  }
+
   // a4..a9: process rates from the post-activation state
   static __device__ __forceinline__ void rates(const ConstK<R> &K, const W<R> &w, double dt, Rt<R> &r) {
     const R T = w.T, p = w.p, rho = w.rho, qv = w.qv, qc = w.qc, qr = w.qr, nc = w.nc, nr = w.nr;
@@ -545,10 +561,22 @@ struct Phys {
     const bool nucl = M::kMixed ? tc < K.tnuc0 : T < K.Tnuc;
 
     // air properties shared by the ventilated integrals
-    const R lgrho = M::lg(rho);
-    const R dfac = M::ex((R)0.4 * (K.lgrho0 - lgrho));         // (rho0/rho)^0.4
-    const R nu = M::div(K.mu_air, rho);
-    const R V0 = M::cbrt(nu * K.inv_dv) * M::sqrt(M::div(dfac, nu));
+    R dfac, V0;   // (rho0/rho)^0.4, cbrt(nu / Dv) sqrt(dfac / nu)
+    if constexpr (M::kMixed) {
+      const R lgrho = M::lg(rho);
+      dfac = M::ex((R)0.4 * (K.lgrho0 - lgrho));
+      const R nu = M::div(K.mu_air, rho);
+      V0 = M::cbrt(nu * K.inv_dv) * M::sqrt(M::div(dfac, nu));
+    } else {
+      // only where a species is there to need them; V0 as one power of rho
+      dfac = V0 = (R)0;
+      if (hr || w.qx[0] > K.qmin || w.qx[1] > K.qmin || w.qx[2] > K.qmin) {
+        const R lgrho = M::lg(rho);
+        dfac = M::ex((R)0.4 * (K.lgrho0 - lgrho));
+        V0 = M::ex(K.v0_ln - (R)(1.0 / 30.0) * lgrho);
+      }
+      r.dfac = dfac;
+    }
 
     r.aut = r.acc = r.scc = r.scr = r.evr = r.nucn = (R)0;
 #pragma unroll
@@ -556,7 +584,7 @@ struct Phys {
     r.rim[0] = r.rim[1] = (R)0;
 
     const R lgqc = hc ? M::lg(qc) : (R)0;
-    const R lgqr = hr ? M::lg(qr) : (R)0;
+    const R lgqr = (M::kMixed ? hr : hr && hc) ? M::lg(qr) : (R)0;
     if (hc) {
       const R ncc = M::mx(rho * nc * (R)1e-6, K.nc_min);
       r.aut = K.kk_aut * M::ex(K.kk_aut_qc * lgqc + K.kk_aut_nc * M::lg(ncc));
@@ -571,10 +599,10 @@ struct Phys {
         if constexpr (M::kTri) {
           typename Shape3<M>::Sh h;
           Shape3<M>::consts(K, 0, w.mu3[0], h);
-          const R l = Shape3<M>::lglam(h, X, lgqr, nr);
+          const R l = M::kMixed ? Shape3<M>::lglam(h, X, lgqr, nr) : Shape3<M>::lglam(h, X, M::lg(qr), nr);
           iv = rho * qr * (h.ev1 * M::ex(X.ex1 * l) + V0 * h.ev2 * M::ex(X.ex2 * l));
         } else {
-          const R l = lglam(X, lgqr, nr);
+          const R l = M::kMixed ? lglam(X, lgqr, nr) : lglam_q(X, qr, nr);
           iv = rho * qr * (X.ev1 * M::ex(X.ex1 * l) + V0 * X.ev2 * M::ex(X.ex2 * l));
         }
         const R Aw = K.awc * iT2, Bw = M::div(K.rv_dv * T, esl);
@@ -606,7 +634,7 @@ struct Phys {
           if (m > 0 && hc)
             r.rim[m - 1] = Shape3<M>::rim(K, 1 + m, w.mu3[1 + m]) * qc * dfac * rho * w.qx[m] * M::ex(X.exr * l);
         } else {
-          const R l = lglam(X, M::lg(w.qx[m]), w.nx[m]);
+          const R l = lglam_q(X, w.qx[m], w.nx[m]);
           const R iv = rho * w.qx[m] * (X.ev1 * M::ex(X.ex1 * l) + V0 * X.ev2 * M::ex(X.ex2 * l));
           r.dep[m] = X.dep * dfa * iv;
           if (m > 0 && hc) r.rim[m - 1] = X.rim * qc * dfac * rho * w.qx[m] * M::ex(X.exr * l);
@@ -625,7 +653,7 @@ struct Phys {
           const R l = Shape3<M>::lglam(h, X, M::lg(w.qx[m]), w.nx[m]);
           iv = rho * w.qx[m] * (h.ev1 * M::ex(X.ex1 * l) + V0 * h.ev2 * M::ex(X.ex2 * l));
         } else {
-          const R l = lglam(X, M::lg(w.qx[m]), w.nx[m]);
+          const R l = lglam_q(X, w.qx[m], w.nx[m]);
           iv = rho * w.qx[m] * (X.ev1 * M::ex(X.ex1 * l) + V0 * X.ev2 * M::ex(X.ex2 * l));
         }
         r.mlt[m] = M::div(X.mlt * tc * iv, rho);
@@ -667,7 +695,7 @@ struct Phys {
     }
     auto fac = [&](R S, R X) -> R {
       if constexpr (!M::kMixed) {
-        return S * dtr > X ? M::mx(X, (R)0) / (S * dtr) : (R)1;
+        return S * dtr > X ? M::div(M::mx(X, (R)0), S * dtr) : (R)1;
       } else {
         // FP32 factor shrunk by 2^-18 so that the rounded transfers can
         // never take more than the pool holds
@@ -701,10 +729,10 @@ struct Phys {
   }
 
   // fall speeds of sedimenting species x (0..3 = r, i, s, g) at one point
-  static __device__ __forceinline__ void fall_speeds(const ConstK<R> &K, R guard, R lgq, R n, R dfac, int x, R &vq,
+  static __device__ __forceinline__ void fall_speeds(const ConstK<R> &K, R guard, R q, R n, R dfac, int x, R &vq,
                                                      R &vn) {
     const SpeciesK<R> &X = K.sp[1 + x];
-    const R l = lglam(X, lgq, n);
+    const R l = lglam_q(X, q, n);
     const R pw = M::ex(X.exv * l);
     vq = M::mn(M::mn(X.vq * dfac * pw, X.vmax), guard);
     vn = M::mn(M::mn(X.vn * dfac * pw, X.vmax), guard);
@@ -736,18 +764,20 @@ struct F64T {
     const double p = s.p;
     if (!(s.qv > qs0 || s.qc > K.qmin)) return;
     const double T0v = s.T, qv0 = s.qv, qc0 = s.qc;
-    double Tn = T0v, es = es0, qs = qs0;
+    double Tn = T0v, es = es0;
+    const double lv_eps_p = K.lv_cp * K.eps * p;
+#pragma unroll 1
     for (int it = 0; it < 4; ++it) {
-      if (it > 0) {
-        es = P::es_liq(K, Tn - K.T0);
-        qs = P::qsat(K, es, p);
-      }
+      // T rests on q_s to the last bit, so its quotients are rounded as
+      // written; their reciprocals serve the slope
       const double tc = Tn - K.T0;
+      double r1, r2;
+      const double ex = div64_in_range(K.esla * tc, tc + K.eslb, r1);
+      if (it > 0) es = K.esl0 * exp64(ex);
+      const double qs = div64_in_range(K.eps * es, p - K.ome * es, r2);
       const double f = (Tn - T0v) - K.lv_cp * (qv0 - qs);
-      const double des = es * K.esla * K.eslb / ((tc + K.eslb) * (tc + K.eslb));
-      const double den = p - K.ome * es;
-      const double fp = 1.0 + K.lv_cp * (K.eps * p / (den * den) * des);
-      Tn = Tn - f / fp;
+      const double des = es * K.eslab * (r1 * r1);
+      Tn = Tn - div64(f, 1.0 + lv_eps_p * (r2 * r2) * des);
     }
     double dq = K.cp_lv * (Tn - T0v);
     if (dq < -qc0) dq = -qc0;
@@ -761,7 +791,7 @@ struct F64T {
     const double N = s.rho * (s.na + s.nc);
     if (!(N > 0.0)) return;
     const double nact = P::arg_nact(K, N, s.w, s.T, s.p, P::es_liq(K, s.T - K.T0));
-    double dn = nact / s.rho - s.nc;
+    double dn = div64(nact, s.rho) - s.nc;
     if (dn < 0.0) dn = 0.0;
     if (dn > s.na) dn = s.na;
     s.nc += dn;
@@ -772,8 +802,9 @@ struct F64T {
   // mu3, keep3 (triple-moment policies): the shapes the rates used, and a bit
   // per species whose sixth moment was only rescaled (no source), so that its
   // shape is unchanged by the processes
+  // dfac: (rho0/rho)^0.4 where a species was there before the processes, else zero
   static __device__ __forceinline__ void process(const ConstK<double> &K, Pt &s, double dt, double es0, double qs0,
-                                                 double *mu3 = nullptr, unsigned *keep3 = nullptr) {
+                                                 double &dfac, double *mu3 = nullptr, unsigned *keep3 = nullptr) {
     const double qc0 = s.qc;
     satadj(K, s, es0, qs0);
     const double evap = qc0 > s.qc ? qc0 - s.qc : 0.0;
@@ -798,6 +829,7 @@ struct F64T {
     }
     Rt<double> r;
     P::rates(K, w, dt, r);
+    dfac = r.dfac;
     Gt<double> g;
     P::limits(K, w, dt, r, g);
     double qxd[3] = {s.qi, s.qs, s.qg};
@@ -810,27 +842,27 @@ struct F64T {
     if (r.acc * g.rc > 0) s.nc -= g.acc * (r.acc * g.rc) * dt;
     if (r.scc > 0) s.nc -= g.scc * r.scc * dt;
     if (r.scr > 0) s.nr -= g.scr * r.scr * dt;
-    if (r.evr > 0) { tau = g.evr * r.evr * dt; s.qr -= tau; s.qv += tau; s.T += tau * (-K.lv) / K.cp; tau_rv = tau; }
+    if (r.evr > 0) { tau = g.evr * r.evr * dt; s.qr -= tau; s.qv += tau; s.T -= tau * K.lv_cp; tau_rv = tau; }
     if (r.evr * g.rr > 0) s.nr -= g.evr * (r.evr * g.rr) * dt;
-    if (g.nucm > 0) { tau = g.nuc * g.nucm * dt; s.qv -= tau; qxd[0] += tau; s.T += tau * K.ls / K.cp; nuc_q = tau; }
+    if (g.nucm > 0) { tau = g.nuc * g.nucm * dt; s.qv -= tau; qxd[0] += tau; s.T += tau * K.ls_cp; nuc_q = tau; }
     if (r.nucn > 0) { nuc_n = g.nuc * r.nucn * dt; nxd[0] += nuc_n; }
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       if (r.dep[m] >= 0) {
-        if (g.depp[m] > 0) { tau = g.dep[m] * g.depp[m] * dt; s.qv -= tau; qxd[m] += tau; s.T += tau * K.ls / K.cp; }
+        if (g.depp[m] > 0) { tau = g.dep[m] * g.depp[m] * dt; s.qv -= tau; qxd[m] += tau; s.T += tau * K.ls_cp; }
       } else {
-        tau = g.dep[m] * g.sub[m] * dt; qxd[m] -= tau; s.qv += tau; s.T += tau * (-K.ls) / K.cp; sub_q[m] = tau;
+        tau = g.dep[m] * g.sub[m] * dt; qxd[m] -= tau; s.qv += tau; s.T -= tau * K.ls_cp; sub_q[m] = tau;
         if (g.sub[m] * g.rx[m] > 0) nxd[m] -= g.dep[m] * (g.sub[m] * g.rx[m]) * dt;
       }
     }
-    if (r.rim[0] > 0) { tau = g.rs * r.rim[0] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf / K.cp; tau_rim += tau; }
+    if (r.rim[0] > 0) { tau = g.rs * r.rim[0] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
     if (r.rim[0] * g.rc > 0) s.nc -= g.rs * (r.rim[0] * g.rc) * dt;
-    if (r.rim[1] > 0) { tau = g.rg * r.rim[1] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf / K.cp; tau_rim += tau; }
+    if (r.rim[1] > 0) { tau = g.rg * r.rim[1] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
     if (r.rim[1] * g.rc > 0) s.nc -= g.rg * (r.rim[1] * g.rc) * dt;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       if (r.mlt[m] > 0) {
-        tau = g.mlt[m] * r.mlt[m] * dt; qxd[m] -= tau; s.qr += tau; s.T += tau * (-K.lf) / K.cp; melt_q[m] = tau;
+        tau = g.mlt[m] * r.mlt[m] * dt; qxd[m] -= tau; s.qr += tau; s.T -= tau * K.lf_cp; melt_q[m] = tau;
       }
       if (g.nmlt[m] > 0) {
         melt_n[m] = g.mlt[m] * g.nmlt[m] * dt; nxd[m] -= melt_n[m]; s.nr += melt_n[m];
@@ -1742,7 +1774,7 @@ __device__ __forceinline__ void courant(const KArgs &a, const ConstK<typename M:
       R vz;
       Shape3<M>::fall_speeds(K, x, (R)1e30, q, M::lg(q), M::toR(nref(s, x)), M::toR(zref(s, x)), dfac, vq, vn, vz);
     } else {
-      Phys<M>::fall_speeds(K, (R)1e30, M::lg(q), M::toR(nref(s, x)), dfac, x, vq, vn);
+      Phys<M>::fall_speeds(K, (R)1e30, q, M::toR(nref(s, x)), dfac, x, vq, vn);
     }
     cmax[x] = M::mx(cmax[x], M::div(vq * M::toR(a.dt), M::toR(sdz[k])));
   }
@@ -1819,7 +1851,14 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
     const R rho = M::toR(rhod);
     const R dfac = M::ex((R)0.4 * (K.lgrho0 - M::lg(rho)));
     const R near = (R)lim * (R)lt.dzdt_f[k];
+    // a level's change by a flux divergence: the mixed form multiplies by
+    // dts / (rho dz); the FP64 form keeps dts dF / (rho dz), which gives back
+    // exactly what the speed limit lets out where it empties a level
     const R sc = M::kMixed ? M::div(M::toRn(dts), M::toRn(rhod) * M::toRn(dz)) : (R)0;
+    auto change = [&](R dF) -> double {
+      if constexpr (M::kMixed) return M::toD(dF * sc);
+      else return M::div(dts * dF, rhod * dz);
+    };
     bool wq = false, we = false;
     inflow = false;
     for (int st = 0; st < ns; ++st) {
@@ -1830,7 +1869,7 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
         if (tri) {
           Shape3<M>::fall_speeds(K, x, (R)1e30, qR, M::lg(qR), M::toR(n), M::toR(e), dfac, vq, vn, vz);
         } else {
-          Ph::fall_speeds(K, (R)1e30, M::lg(qR), M::toR(n), dfac, x, vq, vn);
+          Ph::fall_speeds(K, (R)1e30, qR, M::toR(n), dfac, x, vq, vn);
         }
         if (!(M::mx(M::mx(vq, vn), vz) < near)) {
           const R guard = M::toR(dz / dts);
@@ -1854,21 +1893,15 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
       if (tri || aer) {
         const R X1 = Xu[st];
         if (X != (R)0 || X1 != (R)0) {
-          if constexpr (!M::kMixed) e += dts * (X1 - X) / (rhod * dz);
-          else e += M::toD((X1 - X) * sc);
+          e += change(X1 - X);
           we = true;
           eflag |= nonfinite(e);
         }
         Xu[st] = X;
       }
       if (F != (R)0 || F1 != (R)0 || G != (R)0 || G1 != (R)0) {
-        if constexpr (!M::kMixed) {
-          q += dts * (F1 - F) / (rhod * dz);
-          n += dts * (G1 - G) / (rhod * dz);
-        } else {
-          q += M::toD((F1 - F) * sc);
-          n += M::toD((G1 - G) * sc);
-        }
+        q += change(F1 - F);
+        n += change(G1 - G);
         wq = true;
         eflag |= nonfinite(q) | nonfinite(n);
       }
@@ -2048,7 +2081,7 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
               Shape3<M>::fall_speeds_mu(K, x, guard, lg2a(qpost[x]), n, mus, dfac, vq, vn, vz);
               H = rho * fmaxf(zp, 0.f) * vz;
             } else {
-              Ph::fall_speeds(K, guard, lg2a(qpost[x]), n, dfac, x, vq, vn);
+              Ph::fall_speeds(K, guard, qpost[x], n, dfac, x, vq, vn);
             }
             F = rho * qpost[x] * vq;
             G = rho * fmaxf(n, 0.f) * vn;

@@ -155,13 +155,14 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
         }
         double mu3[4];
         unsigned keep3 = 0;   // species whose shape the processes left unchanged (triple-moment policies)
-        F64T<M>::process(K, s, a.dt, t.es[i], t.qs[i], mu3, &keep3);
+        double dfac;
+        F64T<M>::process(K, s, a.dt, t.es[i], t.qs[i], dfac, mu3, &keep3);
         if (fast) {
           bool any = false;
 #pragma unroll
           for (int x = 0; x < kSed; ++x) any |= qref(s, x) > K.qmin;
           if (any) {
-            const double dfac = ::exp(0.4 * (K.lgrho0 - ::log(s.rho)));
+            if (dfac == 0.0) dfac = exp64(0.4 * (K.lgrho0 - log64(s.rho)));
 #pragma unroll
             for (int x = 0; x < kSed; ++x) {
               const double q = qref(s, x), n = nref(s, x);
@@ -171,10 +172,10 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
                 double vz;
                 const double z = zref(s, x);
                 const double mus = ((keep3 >> x) & 1u) ? mu3[x] : Shape3<M>::mu(K, x, q, n, z);
-                Shape3<M>::fall_speeds_mu(K, x, lt.dzdt[k], ::log(q), n, mus, dfac, vq, vn, vz);
+                Shape3<M>::fall_speeds_mu(K, x, lt.dzdt[k], log64(q), n, mus, dfac, vq, vn, vz);
                 t.flux[kF * x + 2][i] = s.rho * (z > 0.0 ? z : 0.0) * vz;
               } else {
-                Ph::fall_speeds(K, lt.dzdt[k], ::log(q), n, dfac, x, vq, vn);
+                Ph::fall_speeds(K, lt.dzdt[k], q, n, dfac, x, vq, vn);
               }
               t.flux[kF * x][i] = s.rho * q * vq;
               t.flux[kF * x + 1][i] = s.rho * (n > 0.0 ? n : 0.0) * vn;
@@ -215,9 +216,8 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
         const bool act = t.cls[i] != 0;
         double *out = kTend ? tend : a.fld;
         const double *in = kTend && act ? tend : a.fld;   // where the processed values are
-        double rho = 0.0;
-        const double dzk = lt.dz[k];
-        bool have = false;   // rho read: some species moves here
+        double sc = 0.0;     // dt / (rho dz)
+        bool have = false;   // some species moves here
 #pragma unroll
         for (int x = 0; x < kSed; ++x) {
           const double F = t.flux[kF * x][i], F1 = t.flux[kF * x][i - kF64Cols];
@@ -230,7 +230,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
           }
           const bool wx = fast && (X != 0.0 || X1 != 0.0);
           if ((wq || wx) && !have) {
-            rho = __ldg(a.fld + 14 * fs + o);
+            sc = div64(a.dt, __ldg(a.fld + 14 * fs + o) * lt.dz[k]);
             have = true;
           }
           // field 16 + x: a sixth moment; 18 + x: an aerosol mass (source-term row: three less)
@@ -238,8 +238,8 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
           if (wq || kTend) {
             double q = in[(3 + x) * fs + o], n = in[(8 + x) * fs + o];
             if (wq) {
-              q += a.dt * (F1 - F) / (rho * dzk);
-              n += a.dt * (G1 - G) / (rho * dzk);
+              q += (F1 - F) * sc;
+              n += (G1 - G) * sc;
               eflag |= nonfinite(q) | nonfinite(n);
             }
             if (kTend && fast) {
@@ -253,7 +253,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
             if (wx || kTend) {
               double e = in[ix * fs + o];
               if (wx) {
-                e += a.dt * (X1 - X) / (rho * dzk);
+                e += (X1 - X) * sc;
                 eflag |= nonfinite(e);
               }
               if (kTend && fast) e = per_dt(e - a.fld[fx * fs + o]);
