@@ -1637,9 +1637,9 @@ template <class M>
 __host__ __device__ constexpr size_t stage_bytes(int block) {
   return 2 * (size_t)stage_nf<M>() * block * sizeof(double);
 }
-template <class M>
+template <class M, int kB = kBlock>
 __host__ __device__ constexpr size_t step_smem_bytes(int nlev) {
-  return stage_bytes<M>(kBlock) + (size_t)nlev * 24 + (kBlock / 32) * 8;
+  return stage_bytes<M>(kB) + (size_t)nlev * 24 + (kB / 32) * 8;
 }
 
 struct StepSmem {
@@ -1657,9 +1657,9 @@ __device__ __forceinline__ StepSmem level_smem(unsigned char *p, int nlev) {
   m.red = reinterpret_cast<double *>(dzdt_f + nlev);   // 24 nlev bytes in: 8-byte aligned
   return m;
 }
-template <class M>
+template <class M, int kB = kBlock>
 __device__ __forceinline__ StepSmem step_smem(unsigned char *base, int nlev) {
-  StepSmem m = level_smem(base + stage_bytes<M>(kBlock), nlev);
+  StepSmem m = level_smem(base + stage_bytes<M>(kB), nlev);
   m.stage = reinterpret_cast<double *>(base);
   return m;
 }
@@ -2294,7 +2294,7 @@ __host__ __device__ constexpr size_t f64_smem_bytes(int nlev) {
 }
 
 // kTend: tendency mode (tend receives the source terms, a.fld unchanged).
-// Dynamic shared memory: step_smem_bytes<M>(a.nlev), FP64 f64_smem_bytes<M, kStats>(a.nlev).  kStats: the
+// Dynamic shared memory: step_smem_bytes<M, kB>(a.nlev), FP64 f64_smem_bytes<M, kStats>(a.nlev).  kStats: the
 // statistics instantiation (standard configuration; a.stats set).  kLine:
 // whole-line stores for a state in mapped host memory (staged policies).
 //
@@ -2304,8 +2304,10 @@ __host__ __device__ constexpr size_t f64_smem_bytes(int nlev) {
 // of some 4 700 cycles, and one warp per scheduler took 50 of them one after
 // another.  Measured (mixed): 256 columns x 50 levels 114 -> 16 us, 20 000 x 60
 // 172 -> 90 us (step_segments has the line between the two).
-template <class M, bool kTend, bool kStats = false, bool kLine = false, bool kSplit = false>
-__global__ void __launch_bounds__(kBlock, M::kMinBlocks) k_step(const KArgs a, const KParams P, double *tend) {
+//
+// kB: threads per block, kBlock or half of it.
+template <class M, bool kTend, bool kStats = false, bool kLine = false, bool kSplit = false, int kB = kBlock>
+__global__ void __launch_bounds__(kB, M::kMinBlocks * (kBlock / kB)) k_step(const KArgs a, const KParams P, double *tend) {
   extern __shared__ __align__(16) unsigned char step_dyn[];
   ColStats cs{0, 0, {1, 1, 1, 1}};
   unsigned eflag;
@@ -2334,14 +2336,14 @@ __global__ void __launch_bounds__(kBlock, M::kMinBlocks) k_step(const KArgs a, c
     if (c >= a.ncols) return;
     eflag = run_column<M, kTend, kStats, kLine, true>(a, P, sm.lt, fast, c, sg, mine, tend, mine, kBlock, &cs);
   } else {
-    const StepSmem sm = step_smem<M>(step_dyn, a.nlev);
+    const StepSmem sm = step_smem<M, kB>(step_dyn, a.nlev);
     double *mine = sm.stage + threadIdx.x;
-    const int c = blockIdx.x * kBlock + threadIdx.x;
-    if (c < a.ncols) stage_level<M>(a, a.nlev - 1, c, mine, kBlock);
+    const int c = blockIdx.x * kB + threadIdx.x;
+    if (c < a.ncols) stage_level<M>(a, a.nlev - 1, c, mine, kB);
     const bool fast = prologue<false>(a, P, sm, 0, 0);
     if (c >= a.ncols) return;
     eflag = run_column<M, kTend, kStats, kLine, false>(a, P, sm.lt, fast, c, Segment<false>(a.nlev), nullptr, tend, mine,
-                                                       kBlock, &cs);
+                                                       kB, &cs);
   }
   if constexpr (kStats && M::kMixed) stats_add(a.stats, cs);
   if (eflag) atomicOr(a.err, eflag);

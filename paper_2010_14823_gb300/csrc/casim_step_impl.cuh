@@ -26,6 +26,19 @@ inline int step_segments(int ncols, int nlev, int nsm, int blocks_per_sm, bool l
   return n;
 }
 
+// Blocks of half the threads, for a domain of one thread per column that fills
+// no more than one resident wave: its blocks spread unevenly over the SMs
+// (65 536 columns are 3.4 blocks of 128 per SM, so some SMs hold 16 warps and
+// others 12), and the fullest SM sets the time.
+// Measured (65 536 columns): source terms, 150 levels 985 -> 911 us; dt = 10 s,
+// 100 levels 951 -> 929 us; 60 000 x 100 cold 415 -> 412 us; the triple-moment
+// step is bound by its own chain (854 us either way).
+inline bool half_blocks(int warps, int nsm, int blocks_per_sm) {
+  const int whole = (warps + 3) / 4, half = (warps + 1) / 2;
+  if (whole > nsm * blocks_per_sm) return false;
+  return 2 * ((half + nsm - 1) / nsm) < 4 * ((whole + nsm - 1) / nsm);   // warps of the fullest SM
+}
+
 // The FP64 sweep's segments per column group (1 to 8 blocks of a cluster): as
 // many as still fit in one resident wave, at least 4 levels each.
 inline int f64_segments(unsigned groups, int nlev, int nsm, int blocks_per_sm) {
@@ -38,10 +51,10 @@ inline int f64_segments(unsigned groups, int nlev, int nsm, int blocks_per_sm) {
 // grid.x column groups; the levels of a column shared by clusters of grid.y blocks
 template <class K>
 cudaError_t step_launch(K kernel, dim3 grid, size_t smem, cudaStream_t st, const KArgs &a, const KParams &kp,
-                        double *tend) {
+                        double *tend, int block = kBlock) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(kBlock);
+  cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -67,6 +80,8 @@ cudaError_t StepKernels<PMix, PF64>::allow_smem() {
   allow(k_step<PMix, false, false, false, true>, mixed);
   allow(k_step<PMix, true, false, false, true>, mixed);
   allow(k_step<PMix, false, false, true, true>, mixed);
+  allow(k_step<PMix, false, false, false, false, kBlock / 2>, mixed);
+  allow(k_step<PMix, true, false, false, false, kBlock / 2>, mixed);
   allow(k_step<PF64, false>, fp64);
   allow(k_step<PF64, true>, fp64);
   if constexpr (std::is_same<PMix, PolicyMix>::value) {
@@ -99,16 +114,24 @@ cudaError_t StepKernels<PMix, PF64>::launch(const StepLaunch &l, const KArgs &ar
   }
   const int n = step_segments(a.ncols, a.nlev, l.nsm, PMix::kMinBlocks, line);
   const size_t smem = step_smem_bytes<PMix>(a.nlev);
-  auto go = [&](auto *one, auto *split) {
+  const bool half = n == 1 && !line && half_blocks((a.ncols + 31) / 32, l.nsm, PMix::kMinBlocks);
+  auto go = [&](auto *one, auto *split, auto *small) {
+    if (half)
+      return step_launch(small, dim3((unsigned)((a.ncols + kBlock / 2 - 1) / (kBlock / 2))),
+                         step_smem_bytes<PMix, kBlock / 2>(a.nlev), l.stream, a, kp, l.tend, kBlock / 2);
     if (n == 1) return step_launch(one, whole, smem, l.stream, a, kp, l.tend);
     a.segs = n < kBlock / 32 ? n : kBlock / 32;   // a warp per segment in the block, the rest over a cluster
     const int cols = kBlock / a.segs;
     return step_launch(split, dim3((unsigned)((a.ncols + cols - 1) / cols), (unsigned)(n / a.segs)), smem, l.stream, a,
                        kp, l.tend);
   };
-  if (l.tend) return go(k_step<PMix, true>, k_step<PMix, true, false, false, true>);
-  if (line) return go(k_step<PMix, false, false, true>, k_step<PMix, false, false, true, true>);
-  return go(k_step<PMix, false>, k_step<PMix, false, false, false, true>);
+  if (l.tend)
+    return go(k_step<PMix, true>, k_step<PMix, true, false, false, true>,
+              k_step<PMix, true, false, false, false, kBlock / 2>);
+  if (line)
+    return go(k_step<PMix, false, false, true>, k_step<PMix, false, false, true, true>, k_step<PMix, false, false, true>);
+  return go(k_step<PMix, false>, k_step<PMix, false, false, false, true>,
+            k_step<PMix, false, false, false, false, kBlock / 2>);
 }
 
 }  // namespace casim_dev
