@@ -77,8 +77,7 @@ __device__ __forceinline__ bool point_needs_step(const KParams &P, const DomDesc
                          max(max(hiabs(s.qi), hiabs(s.qs)), max(hiabs(s.qg), hiabs(s.p))));
   if (h >= 0x7ff00000u) return true;
   if constexpr (!M::kMixed) {
-    double es0, qs0;
-    return F64::active(P.d, s, es0, qs0);
+    return F64::flag(P.d, P.f, s) != 0;
   } else {
     W<float> w;
     float es0, qs0;

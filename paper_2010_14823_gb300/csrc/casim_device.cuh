@@ -232,6 +232,10 @@ struct PolicyF64 {
   static __device__ __forceinline__ R div(R a, R b) { return div64(a, b); }
   static __device__ __forceinline__ R mn(R a, R b) { return a < b ? a : b; }
   static __device__ __forceinline__ R mx(R a, R b) { return a > b ? a : b; }
+  // a > b for a and b not both negative, on the integer pipe (an FP64 compare
+  // costs as much as an addition): IEEE values of that kind order as their bits
+  static __device__ __forceinline__ bool gt(R a, R b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+  static __device__ __forceinline__ R pos(R a) { return __double2hiint(a) < 0 ? 0.0 : a; }   // max(a, 0)
 };
 
 struct PolicyMix {
@@ -273,6 +277,8 @@ struct PolicyMix {
   static __device__ __forceinline__ R div(R a, R b) { return __fdividef(a, b); }
   static __device__ __forceinline__ R mn(R a, R b) { return fminf(a, b); }
   static __device__ __forceinline__ R mx(R a, R b) { return fmaxf(a, b); }
+  static __device__ __forceinline__ bool gt(R a, R b) { return a > b; }
+  static __device__ __forceinline__ R pos(R a) { return fmaxf(a, 0.f); }
 };
 
 // ------------------------------------------------------------ one point
@@ -536,7 +542,7 @@ struct Phys {
     if constexpr (M::kMixed) {
       return lglam(X, M::lg(q), n);
     } else {
-      R l = (X.lglamfac + M::lg(M::div(M::mx(n, (R)0), q))) * X.invb;
+      R l = (X.lglamfac + M::lg(M::div(M::pos(n), q))) * X.invb;
       l = M::mx(l, X.lglo);
       return M::mn(l, X.lghi);
     }
@@ -551,7 +557,7 @@ struct Phys {
     const R qsl = qsat(K, esl, p);
     const R iT2 = M::div((R)1, T * T);
     const R Sw = M::div(qv, qsl);
-    const bool hc = qc > K.qmin, hr = qr > K.qmin;
+    const bool hc = M::gt(qc, K.qmin), hr = M::gt(qr, K.qmin);
     // regimes: the FP64 form compares T itself; the mixed form compares
     // tc = T - T0, which it forms in FP64 before rounding (an FP32 T is
     // resolved to 3e-5 K only, so a point adjusted to within that of the
@@ -570,7 +576,7 @@ struct Phys {
     } else {
       // only where a species is there to need them; V0 as one power of rho
       dfac = V0 = (R)0;
-      if (hr || w.qx[0] > K.qmin || w.qx[1] > K.qmin || w.qx[2] > K.qmin) {
+      if (hr || M::gt(w.qx[0], K.qmin) || M::gt(w.qx[1], K.qmin) || M::gt(w.qx[2], K.qmin)) {
         const R lgrho = M::lg(rho);
         dfac = M::ex((R)0.4 * (K.lgrho0 - lgrho));
         V0 = M::ex(K.v0_ln - (R)(1.0 / 30.0) * lgrho);
@@ -592,7 +598,7 @@ struct Phys {
     }
     if (hc && hr) r.acc = K.kk_acc * M::ex(K.kk_acc_exp * (lgqc + lgqr));
     if (hr) {
-      r.scr = K.kr * rho * M::mx(nr, (R)0) * qr;
+      r.scr = K.kr * rho * M::pos(nr) * qr;
       if (Sw < (R)1) {
         const SpeciesK<R> &X = K.sp[1];
         R iv;
@@ -622,7 +628,7 @@ struct Phys {
       const R dfa = M::div(Si - (R)1, rho * (Ai + Bi));
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
-        if (!(w.qx[m] > K.qmin)) continue;
+        if (!M::gt(w.qx[m], K.qmin)) continue;
         const SpeciesK<R> &X = K.sp[2 + m];
         if constexpr (M::kTri) {
           // at the species' diagnosed shape
@@ -644,7 +650,7 @@ struct Phys {
     if (!M::kWarm && warm) {
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
-        if (!(w.qx[m] > K.qmin)) continue;
+        if (!M::gt(w.qx[m], K.qmin)) continue;
         const SpeciesK<R> &X = K.sp[2 + m];
         R iv;
         if constexpr (M::kTri) {
@@ -667,16 +673,16 @@ struct Phys {
   static __device__ __forceinline__ void limits(const ConstK<R> &K, const W<R> &w, double dt, const Rt<R> &r,
                                                 Gt<R> &g) {
     const R dtr = M::toR(dt);
-    g.rc = w.qc > K.qmin ? M::div(M::mx(w.nc, (R)0), w.qc) : (R)0;
-    g.rr = w.qr > K.qmin ? M::div(M::mx(w.nr, (R)0), w.qr) : (R)0;
+    g.rc = M::gt(w.qc, K.qmin) ? M::div(M::pos(w.nc), w.qc) : (R)0;
+    g.rr = M::gt(w.qr, K.qmin) ? M::div(M::pos(w.nr), w.qr) : (R)0;
 #pragma unroll
-    for (int m = 0; m < 3; ++m) g.rx[m] = w.qx[m] > K.qmin ? M::div(M::mx(w.nx[m], (R)0), w.qx[m]) : (R)0;
+    for (int m = 0; m < 3; ++m) g.rx[m] = M::gt(w.qx[m], K.qmin) ? M::div(M::pos(w.nx[m]), w.qx[m]) : (R)0;
     g.nucm = r.nucn * K.mi0;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       g.depp[m] = r.dep[m] >= (R)0 ? r.dep[m] : (R)0;
       g.sub[m] = r.dep[m] >= (R)0 ? (R)0 : -r.dep[m];
-      g.nmlt[m] = r.mlt[m] > (R)0 ? r.mlt[m] * g.rx[m] : (R)0;
+      g.nmlt[m] = M::gt(r.mlt[m], (R)0) ? r.mlt[m] * g.rx[m] : (R)0;
     }
     // sinks per pool, summed in the order of the transfer list
     const R S_qv = ((g.nucm + g.depp[0]) + g.depp[1]) + g.depp[2];
@@ -695,7 +701,7 @@ struct Phys {
     }
     auto fac = [&](R S, R X) -> R {
       if constexpr (!M::kMixed) {
-        return S * dtr > X ? M::div(M::mx(X, (R)0), S * dtr) : (R)1;
+        return M::gt(S * dtr, X) ? M::div(M::pos(X), S * dtr) : (R)1;
       } else {
         // FP32 factor shrunk by 2^-18 so that the rounded transfers can
         // never take more than the pool holds
@@ -707,8 +713,8 @@ struct Phys {
     const R f_nc = fac(S_nc, w.nc), f_nr = fac(S_nr, w.nr);
     auto g2 = [&](R rate, R fm, R nsink, R fn) -> R {
       R x = (R)1;
-      if (rate > (R)0 && fm < x) x = fm;
-      if (nsink > (R)0 && fn < x) x = fn;
+      if (M::gt(rate, (R)0) && M::gt(x, fm)) x = fm;
+      if (M::gt(nsink, (R)0) && M::gt(x, fn)) x = fn;
       return x;
     };
     g.aut = g2(r.aut, f_qc, r.aut * g.rc, f_nc);
@@ -744,27 +750,45 @@ template <class M>
 struct F64T {
   using P = Phys<M>;
 
-  // true unless the chain leaves the point unchanged (no hydrometeor, not
-  // supersaturated over liquid, no ice nucleation possible); also returns
-  // q_s over liquid at the initial temperature for the adjustment
-  static __device__ __forceinline__ bool active(const ConstK<double> &K, const Pt &s, double &es0, double &qs0) {
-    const double qmin = K.qmin;
-    es0 = P::es_liq(K, s.T - K.T0);
-    qs0 = P::qsat(K, es0, s.p);
-    bool act = s.qc > qmin || s.qr > qmin || s.qv > qs0;
-    if constexpr (!M::kWarm) {
-      act = act || s.qi > qmin || s.qs > qmin || s.qg > qmin;
-      if (!act && s.T < K.Tnuc) act = s.qv / P::qsat(K, P::es_ice(K, s.T, 0.0), s.p) > 1.0;
+  // q > q_s(T, p) over liquid (ice: over ice).  Decided in FP32 where the two
+  // differ by more than 1e-4 of q_s (the FP32 value is good to ~2e-6), else by
+  // the FP64 expression.
+  template <bool kIce>
+  static __device__ __forceinline__ bool supersaturated(const ConstK<double> &K, const ConstK<float> &Kf, const Pt &s) {
+    if (max(max(hiabs(s.T), hiabs(s.p)), hiabs(s.qv)) < kF32RangeHi) {
+      const float T = d2f(s.T), p = d2f(s.p), q = d2f(s.qv);
+      const float tc = T - Kf.T0;
+      const float es = kIce ? Kf.esi0 * PolicyMix::exp(__fdividef(Kf.esia * (T - Kf.esit), T - Kf.esib))
+                            : Kf.esl0 * PolicyMix::exp(__fdividef(Kf.esla * tc, tc + Kf.eslb));
+      const float qs = __fdividef(Kf.eps * es, p - Kf.ome * es);
+      if (qs > 0.f) {
+        if (q > 1.0001f * qs) return true;
+        if (q < 0.9999f * qs) return false;
+      }
     }
-    return act;
+    if constexpr (kIce) return s.qv / P::qsat(K, P::es_ice(K, s.T, 0.0), s.p) > 1.0;
+    else return s.qv > P::qsat(K, P::es_liq(K, s.T - K.T0), s.p);
+  }
+
+  // 0 unless the chain can change the point (a hydrometeor, supersaturated
+  // over liquid, or ice nucleation possible); 1: by adjustment too, below T0;
+  // 2: so, above; 3: not by adjustment
+  static __device__ __forceinline__ unsigned flag(const ConstK<double> &K, const ConstK<float> &Kf, const Pt &s) {
+    const bool adj = M::gt(s.qc, K.qmin) || supersaturated<false>(K, Kf, s);
+    if (adj) return M::gt(K.T0, s.T) ? 1 : 2;
+    bool act = M::gt(s.qr, K.qmin);
+    if constexpr (!M::kWarm) {
+      act = act || M::gt(s.qi, K.qmin) || M::gt(s.qs, K.qmin) || M::gt(s.qg, K.qmin);
+      act = act || (M::gt(K.Tnuc, s.T) && supersaturated<true>(K, Kf, s));
+    }
+    return act ? 3 : 0;
   }
 
   // a2: 4 Newton iterations on cp (T* - T) = Lv (qv - qs(T*))
-  static __device__ __forceinline__ void satadj(const ConstK<double> &K, Pt &s, double es0, double qs0) {
+  static __device__ __forceinline__ void satadj(const ConstK<double> &K, Pt &s) {
     const double p = s.p;
-    if (!(s.qv > qs0 || s.qc > K.qmin)) return;
     const double T0v = s.T, qv0 = s.qv, qc0 = s.qc;
-    double Tn = T0v, es = es0;
+    double Tn = T0v;
     const double lv_eps_p = K.lv_cp * K.eps * p;
 #pragma unroll 1
     for (int it = 0; it < 4; ++it) {
@@ -773,7 +797,7 @@ struct F64T {
       const double tc = Tn - K.T0;
       double r1, r2;
       const double ex = div64_in_range(K.esla * tc, tc + K.eslb, r1);
-      if (it > 0) es = K.esl0 * exp64(ex);
+      const double es = K.esl0 * exp64(ex);
       const double qs = div64_in_range(K.eps * es, p - K.ome * es, r2);
       const double f = (Tn - T0v) - K.lv_cp * (qv0 - qs);
       const double des = es * K.eslab * (r1 * r1);
@@ -787,9 +811,9 @@ struct F64T {
   }
 
   static __device__ __forceinline__ void activate(const ConstK<double> &K, Pt &s) {
-    if (!(s.w > 0.0) || !(s.qc > K.qmin)) return;
+    if (!M::gt(s.w, 0.0) || !M::gt(s.qc, K.qmin)) return;
     const double N = s.rho * (s.na + s.nc);
-    if (!(N > 0.0)) return;
+    if (!M::gt(N, 0.0)) return;
     const double nact = P::arg_nact(K, N, s.w, s.T, s.p, P::es_liq(K, s.T - K.T0));
     double dn = div64(nact, s.rho) - s.nc;
     if (dn < 0.0) dn = 0.0;
@@ -803,10 +827,11 @@ struct F64T {
   // per species whose sixth moment was only rescaled (no source), so that its
   // shape is unchanged by the processes
   // dfac: (rho0/rho)^0.4 where a species was there before the processes, else zero
-  static __device__ __forceinline__ void process(const ConstK<double> &K, Pt &s, double dt, double es0, double qs0,
-                                                 double &dfac, double *mu3 = nullptr, unsigned *keep3 = nullptr) {
+  // adjust: qv > q_s or cloud is present (flag() < 3)
+  static __device__ __forceinline__ void process(const ConstK<double> &K, Pt &s, double dt, bool adjust, double &dfac,
+                                                 double *mu3 = nullptr, unsigned *keep3 = nullptr) {
     const double qc0 = s.qc;
-    satadj(K, s, es0, qs0);
+    if (adjust) satadj(K, s);
     const double evap = qc0 > s.qc ? qc0 - s.qc : 0.0;
     const double na1 = s.na;
     activate(K, s);
@@ -835,36 +860,36 @@ struct F64T {
     double qxd[3] = {s.qi, s.qs, s.qg};
     double nxd[3] = {s.ni, s.ns, s.ng};
     double tau;
-    if (r.aut > 0) { tau = g.aut * r.aut * dt; s.qc -= tau; s.qr += tau; tau_cr += tau; tau_aut = tau; }
-    if (r.aut * g.rc > 0) s.nc -= g.aut * (r.aut * g.rc) * dt;
-    if (r.aut * K.inv_mr0 > 0) { nr_aut = g.aut * (r.aut * K.inv_mr0) * dt; s.nr += nr_aut; }
-    if (r.acc > 0) { tau = g.acc * r.acc * dt; s.qc -= tau; s.qr += tau; tau_cr += tau; }
-    if (r.acc * g.rc > 0) s.nc -= g.acc * (r.acc * g.rc) * dt;
-    if (r.scc > 0) s.nc -= g.scc * r.scc * dt;
-    if (r.scr > 0) s.nr -= g.scr * r.scr * dt;
-    if (r.evr > 0) { tau = g.evr * r.evr * dt; s.qr -= tau; s.qv += tau; s.T -= tau * K.lv_cp; tau_rv = tau; }
-    if (r.evr * g.rr > 0) s.nr -= g.evr * (r.evr * g.rr) * dt;
-    if (g.nucm > 0) { tau = g.nuc * g.nucm * dt; s.qv -= tau; qxd[0] += tau; s.T += tau * K.ls_cp; nuc_q = tau; }
-    if (r.nucn > 0) { nuc_n = g.nuc * r.nucn * dt; nxd[0] += nuc_n; }
+    if (M::gt(r.aut, 0.0)) { tau = g.aut * r.aut * dt; s.qc -= tau; s.qr += tau; tau_cr += tau; tau_aut = tau; }
+    if (M::gt(r.aut * g.rc, 0.0)) s.nc -= g.aut * (r.aut * g.rc) * dt;
+    if (M::gt(r.aut * K.inv_mr0, 0.0)) { nr_aut = g.aut * (r.aut * K.inv_mr0) * dt; s.nr += nr_aut; }
+    if (M::gt(r.acc, 0.0)) { tau = g.acc * r.acc * dt; s.qc -= tau; s.qr += tau; tau_cr += tau; }
+    if (M::gt(r.acc * g.rc, 0.0)) s.nc -= g.acc * (r.acc * g.rc) * dt;
+    if (M::gt(r.scc, 0.0)) s.nc -= g.scc * r.scc * dt;
+    if (M::gt(r.scr, 0.0)) s.nr -= g.scr * r.scr * dt;
+    if (M::gt(r.evr, 0.0)) { tau = g.evr * r.evr * dt; s.qr -= tau; s.qv += tau; s.T -= tau * K.lv_cp; tau_rv = tau; }
+    if (M::gt(r.evr * g.rr, 0.0)) s.nr -= g.evr * (r.evr * g.rr) * dt;
+    if (M::gt(g.nucm, 0.0)) { tau = g.nuc * g.nucm * dt; s.qv -= tau; qxd[0] += tau; s.T += tau * K.ls_cp; nuc_q = tau; }
+    if (M::gt(r.nucn, 0.0)) { nuc_n = g.nuc * r.nucn * dt; nxd[0] += nuc_n; }
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       if (r.dep[m] >= 0) {
-        if (g.depp[m] > 0) { tau = g.dep[m] * g.depp[m] * dt; s.qv -= tau; qxd[m] += tau; s.T += tau * K.ls_cp; }
+        if (M::gt(g.depp[m], 0.0)) { tau = g.dep[m] * g.depp[m] * dt; s.qv -= tau; qxd[m] += tau; s.T += tau * K.ls_cp; }
       } else {
         tau = g.dep[m] * g.sub[m] * dt; qxd[m] -= tau; s.qv += tau; s.T -= tau * K.ls_cp; sub_q[m] = tau;
-        if (g.sub[m] * g.rx[m] > 0) nxd[m] -= g.dep[m] * (g.sub[m] * g.rx[m]) * dt;
+        if (M::gt(g.sub[m] * g.rx[m], 0.0)) nxd[m] -= g.dep[m] * (g.sub[m] * g.rx[m]) * dt;
       }
     }
-    if (r.rim[0] > 0) { tau = g.rs * r.rim[0] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
-    if (r.rim[0] * g.rc > 0) s.nc -= g.rs * (r.rim[0] * g.rc) * dt;
-    if (r.rim[1] > 0) { tau = g.rg * r.rim[1] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
-    if (r.rim[1] * g.rc > 0) s.nc -= g.rg * (r.rim[1] * g.rc) * dt;
+    if (M::gt(r.rim[0], 0.0)) { tau = g.rs * r.rim[0] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
+    if (M::gt(r.rim[0] * g.rc, 0.0)) s.nc -= g.rs * (r.rim[0] * g.rc) * dt;
+    if (M::gt(r.rim[1], 0.0)) { tau = g.rg * r.rim[1] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
+    if (M::gt(r.rim[1] * g.rc, 0.0)) s.nc -= g.rg * (r.rim[1] * g.rc) * dt;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      if (r.mlt[m] > 0) {
+      if (M::gt(r.mlt[m], 0.0)) {
         tau = g.mlt[m] * r.mlt[m] * dt; qxd[m] -= tau; s.qr += tau; s.T -= tau * K.lf_cp; melt_q[m] = tau;
       }
-      if (g.nmlt[m] > 0) {
+      if (M::gt(g.nmlt[m], 0.0)) {
         melt_n[m] = g.mlt[m] * g.nmlt[m] * dt; nxd[m] -= melt_n[m]; s.nr += melt_n[m];
       }
     }

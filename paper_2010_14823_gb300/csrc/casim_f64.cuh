@@ -13,16 +13,31 @@
 // point alone, so only the update needs the level above.
 // Measured: FP64 step, 256x256x100 stratus 28.7 -> 9.9 ms (24.7 lanes, FP64
 // pipe 66 % busy over the launch instead of 45 %), deep convection of that size
-// 35.5 -> 16.9 ms, 2 000 columns 5.2 -> 0.52 ms.
+// 35.5 -> 16.9 ms, 2 000 columns 5.2 -> 0.52 ms; with the functions of
+// casim_math64.cuh 6.2, 10.5 and 0.36 ms; with the flags decided in FP32 away
+// from saturation and comparisons on the integer pipe (an FP64 compare costs as
+// much as an addition) 4.9, 8.7 and 0.30 ms, bit for bit the same.
 // (included by casim_device.cuh)
 #pragma once
 
 namespace casim_dev {
 
 constexpr int kF64Cols = 32;      // columns of a tile
-constexpr int kF64Levels = 16;    // levels of a chunk
-constexpr int kF64Pts = (kF64Levels + 1) * kF64Cols;   // row 0: the level above the chunk
+// levels of a chunk: as many as leave three blocks to an SM (8 fluxes a point
+// at 32 levels; 16 levels where points hand down 12).  Measured, cold step,
+// 8 / 16 / 24 / 32 levels: 6.46 / 6.18 / 6.07 / 6.04 ms
+template <class M>
+__host__ __device__ constexpr int f64_levels() {
+  return M::kWarm || M::kTri || M::kAero ? 16 : 32;
+}
+template <class M>
+__host__ __device__ constexpr int f64_points() {   // row 0: the level above the chunk
+  return (f64_levels<M>() + 1) * kF64Cols;
+}
 constexpr int kF64Classes = 3;
+
+// x != 0 on the integer pipe
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) & 0x7fffffffffffffffll) != 0; }
 
 // flux arrays: mass and number of each sedimenting species, and its sixth
 // moment or aerosol mass
@@ -33,14 +48,14 @@ __host__ __device__ constexpr int f64_fluxes() {
 
 template <class M>
 struct F64Tile {
-  double flux[f64_fluxes<M>()][kF64Pts];
-  double es[kF64Pts], qs[kF64Pts];              // saturation at the initial temperature
+  static constexpr int kPts = f64_points<M>();
+  double flux[f64_fluxes<M>()][kPts];
   double halo[22][kF64Cols];                    // the level above the segment, as read
   unsigned long long cmax[4][kF64Cols];         // multi-substep path: largest Courant numbers (bits)
   int cnt[kF64Classes + 1];
   int col[kF64Cols];                            // the tile's columns, -1: none
-  unsigned short list[kF64Pts];                 // active points, by class
-  unsigned char cls[kF64Pts];                   // 0: inactive, else 1 + class
+  unsigned short list[kPts];                 // active points, by class
+  unsigned char cls[kPts];                   // 0: inactive, else 1 + class
 };
 
 // Statistics of a tile's columns (the statistics instantiation).
@@ -76,9 +91,9 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
       for (unsigned &w : st->lv[i]) w = 0u;
     }
   }
-  for (int ktop = sg.ktop(); ktop >= sg.kbot(); ktop -= kF64Levels) {
+  for (int ktop = sg.ktop(); ktop >= sg.kbot(); ktop -= f64_levels<M>()) {
     const bool first = ktop == sg.ktop();
-    const int rows = 1 + min(kF64Levels, ktop - sg.kbot() + 1);
+    const int rows = 1 + min(f64_levels<M>(), ktop - sg.kbot() + 1);
     const int i0 = first && halo ? 0 : kF64Cols, i1 = rows * kF64Cols;   // this chunk's points
     if (tid <= kF64Classes) t.cnt[tid] = 0;
     __syncthreads();
@@ -96,12 +111,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
 #pragma unroll
           for (int f = 0; f < 16 + nextra<M>(); ++f) t.halo[f][lane] = pt_field<M>(s, f);
         }
-        double es0, qs0;
-        if (F64T<M>::active(K, s, es0, qs0)) {
-          t.es[i] = es0;
-          t.qs[i] = qs0;
-          cls = !(s.qv > qs0 || s.qc > K.qmin) ? 3 : s.T < K.T0 ? 1 : 2;
-        }
+        cls = F64T<M>::flag(K, P.f, s);
       }
       t.cls[i] = (unsigned char)cls;
       if constexpr (kStats) {
@@ -156,17 +166,17 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
         double mu3[4];
         unsigned keep3 = 0;   // species whose shape the processes left unchanged (triple-moment policies)
         double dfac;
-        F64T<M>::process(K, s, a.dt, t.es[i], t.qs[i], dfac, mu3, &keep3);
+        F64T<M>::process(K, s, a.dt, t.cls[i] < 3, dfac, mu3, &keep3);
         if (fast) {
           bool any = false;
 #pragma unroll
-          for (int x = 0; x < kSed; ++x) any |= qref(s, x) > K.qmin;
+          for (int x = 0; x < kSed; ++x) any |= M::gt(qref(s, x), K.qmin);
           if (any) {
             if (dfac == 0.0) dfac = exp64(0.4 * (K.lgrho0 - log64(s.rho)));
 #pragma unroll
             for (int x = 0; x < kSed; ++x) {
               const double q = qref(s, x), n = nref(s, x);
-              if (!(q > K.qmin)) continue;
+              if (!M::gt(q, K.qmin)) continue;
               double vq, vn;
               if (x < nz3<M>()) {
                 double vz;
@@ -178,7 +188,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
                 Ph::fall_speeds(K, lt.dzdt[k], q, n, dfac, x, vq, vn);
               }
               t.flux[kF * x][i] = s.rho * q * vq;
-              t.flux[kF * x + 1][i] = s.rho * (n > 0.0 ? n : 0.0) * vn;
+              t.flux[kF * x + 1][i] = s.rho * M::pos(n) * vn;
               if (x < na3<M>()) t.flux[kF * x + 2][i] = s.rho * maref(s, x) * vq;
             }
           }
@@ -222,13 +232,13 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
         for (int x = 0; x < kSed; ++x) {
           const double F = t.flux[kF * x][i], F1 = t.flux[kF * x][i - kF64Cols];
           const double G = t.flux[kF * x + 1][i], G1 = t.flux[kF * x + 1][i - kF64Cols];
-          const bool wq = fast && (F != 0.0 || F1 != 0.0 || G != 0.0 || G1 != 0.0);
+          const bool wq = fast && (nonzero(F) || nonzero(F1) || nonzero(G) || nonzero(G1));
           double X = 0.0, X1 = 0.0;
           if constexpr (kF == 3) {
             X = t.flux[kF * x + 2][i];
             X1 = t.flux[kF * x + 2][i - kF64Cols];
           }
-          const bool wx = fast && (X != 0.0 || X1 != 0.0);
+          const bool wx = fast && (nonzero(X) || nonzero(X1));
           if ((wq || wx) && !have) {
             sc = div64(a.dt, __ldg(a.fld + 14 * fs + o) * lt.dz[k]);
             have = true;
