@@ -720,27 +720,31 @@ namespace casim_dev {
 
 // Weight images in global memory, already in the swizzled shared-memory
 // layout, so that 1-D bulk copies land them ready for the tensor cores:
-//   W1: [256 rows][64] (k >= 12 zero)                                32 KB
-//   W2, W3: four chunks each, chunk s = all 256 output rows x k = 64s..64s+63
-//           (one K-slab)                                              32 KB each
+//   W1: [256 rows][16] (k >= 12 zero), 32-byte swizzle               8 KB
+//   W2, W3: per K-step of 16 an image like W1's, 16 steps each      8 KB a step
 //   W4: [16 rows][256] (rows >= 4 zero)                               8 KB
-constexpr uint32_t kImgW1 = 256 * 128, kImgChunk = 256 * 128, kImgW4 = 16 * 4 * 128;
-constexpr int kImgChunks = 8;
+// K-steps per ring stage: two (16 KB, four stages).  On the rows stated at the
+// kernel: 1020 us with two, 1090 with four (two stages only: a copy of
+// 32 KB is not covered), 1440 with one (a wait and a commit for every MMA).
+constexpr int kUmmaSteps = 2;
+constexpr uint32_t kImgStep = 256 * 32;
+constexpr uint32_t kImgW1 = 256 * 32, kImgChunk = kUmmaSteps * kImgStep, kImgW4 = 16 * 4 * 128;
+constexpr int kImgChunks = 32 / kUmmaSteps;
 constexpr uint32_t kImgBytes = kImgW1 + kImgChunks * kImgChunk + kImgW4;
 
 __global__ void k_mlp_images(const float *theta, unsigned char *img) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const __nv_bfloat16 z = __float2bfloat16(0.f);
-  if (i < 256 * 64) {   // W1 (n, k)
-    const int n = i / 64, k = i % 64;
-    *reinterpret_cast<__nv_bfloat16 *>(img + sw128_offset(256, n, k)) =
+  if (i < 256 * 16) {   // W1 (n, k)
+    const int n = i / 16, k = i % 16;
+    *reinterpret_cast<__nv_bfloat16 *>(img + sw32_offset(n, k)) =
         k < kNin ? __float2bfloat16(theta[kOffW1 + k * kNh + n]) : z;
   }
   if (i < 256 * 256) {  // W2, W3 (n, k)
-    const int n = i / 256, k = i % 256, s = k >> 6;
-    const uint32_t off = (uint32_t)s * kImgChunk + sw128_offset(256, n, k & 63);
+    const int n = i / 256, k = i % 256;
+    const uint32_t off = (uint32_t)(k >> 4) * kImgStep + sw32_offset(n, k & 15);
     *reinterpret_cast<__nv_bfloat16 *>(img + kImgW1 + off) = __float2bfloat16(theta[kOffW2 + k * kNh + n]);
-    *reinterpret_cast<__nv_bfloat16 *>(img + kImgW1 + 4 * kImgChunk + off) = __float2bfloat16(theta[kOffW3 + k * kNh + n]);
+    *reinterpret_cast<__nv_bfloat16 *>(img + kImgW1 + 16 * kImgStep + off) = __float2bfloat16(theta[kOffW3 + k * kNh + n]);
   }
   if (i < 16 * 256) {   // W4 (n, k)
     const int n = i / 256, k = i % 256;
@@ -768,39 +772,36 @@ constexpr int kUmmaEpiWarps = 16;                       // 4 per TMEM lane quart
 constexpr int kUmmaMmaWarp = kUmmaEpiWarps;             // issues the MMAs, owns TMEM
 constexpr int kUmmaProdWarp = kUmmaEpiWarps + 1;        // streams the weight chunks
 constexpr int kUmmaThreads = (kUmmaEpiWarps + 2) * 32;
-constexpr int kUmmaStages = 4;                          // weight-chunk ring
-// dynamic shared memory (1024-byte aligned): resident W1 and W4, the chunk
-// ring.  Activations live in tensor memory.
-constexpr uint32_t kSmW1 = 0, kSmW4 = kSmW1 + kImgW1, kSmRing = kSmW4 + kImgW4;
-// tensor-memory columns: accumulators A0 (layers 1, 3) and A1 (layers 2, 4),
-// each later overwritten in place by its layer's BF16 activations; the next
-// tile's features sit in A1's last 8 columns
-constexpr uint32_t kTmA0 = 0, kTmA1 = 256, kTmFeat = 504;
+constexpr int kUmmaStages = 8 / kUmmaSteps;                          // weight-chunk ring
+// dynamic shared memory (1024-byte aligned): resident W1 and W4, the features
+// and activations of two tiles, the chunk ring
+constexpr uint32_t kUmmaFeat = 128 * 32, kUmmaAct = 4 * 128 * 128;
+constexpr uint32_t kSmW1 = 0, kSmW4 = kSmW1 + kImgW1, kSmFeat = kSmW4 + kImgW4, kSmAct = kSmFeat + 2 * kUmmaFeat,
+                   kSmRing = kSmAct + 2 * kUmmaAct;
 constexpr int kUmmaSmem = 1024 + kSmRing + kUmmaStages * kImgChunk;
 static_assert(kUmmaSmem + 4096 <= 232448, "shared memory of the tensor-core kernel");
 
-// Persistent, one CTA (18 warps) per SM, 128-row tiles.
+// Persistent, one CTA (18 warps) per SM, 128-row tiles, two in flight.
 //
-// Tensor memory holds two 256-column FP32 accumulators used by alternate
-// layers (layer 1 -> A0, 2 -> A1, 3 -> A0, 4 -> A1), so the MMAs of layer
-// l+1 run while the epilogue of layer l still reads layer l's sums.  The
-// activations never touch shared memory: each epilogue warp writes the BF16
-// activations of the 16 sums it has just read back into the first 8 of
-// those 16 columns (two per 32-bit column, even k in the low half), and the
-// next layer's MMAs read their A operand from there (K-step kk of 16 at
-// column 16 kk).  Shared memory only holds weights, and its bandwidth --
-// which bounds these MMAs -- goes to the B operand:
-//  * epilogue warps (16): warp w reads TMEM lanes 32(w%4).. (its rows) and
-//    columns 16(w/4)..+15 of each 64-column slab; per slab s: bias, tanh,
-//    BF16 pack, tcgen05.st in place, then one arrival on act[s];
-//  * MMA warp (one thread): per slab s it waits act[s] and issues that
-//    K-slab's MMAs of the next layer (N = 256, weights from the ring);
-//    after the last slab it commits the accumulator to acc;
-//  * producer warp (one thread): streams the 8 weight chunks of layers 2-3
-//    per tile through the ring (full/free barriers).
-// Weight traffic from L2 is 256 KB per tile.  N = 256 MMAs read each A slab once
-// (N = 128 halves would read it twice): shared-memory operand bandwidth, not
-// the tensor pipe, bounds these MMAs.
+// What bounds it is tanh: 98 304 per 128-row tile at 16 per SM and clock are
+// 6.1 k cycles; the MMAs need 4.4 k.  Each tile has a 256-column FP32
+// accumulator of its own in tensor memory; the BF16 activations go to shared
+// memory, so that the next layer's sums can replace this layer's in the same
+// columns.  While the epilogue warps work on one tile's layer, the other
+// tile's next layer is multiplied:
+//  * epilogue warps (16): for each layer, tile by tile, warp w reads lanes
+//    32(w%4).. (its rows) and the 64 columns of slab w/4: bias, tanh, BF16
+//    pack, to the activation slab; then one arrival on the tile's act barrier;
+//  * MMA warp (one thread): once a tile's activations are complete, the next
+//    layer's MMAs (N = 256, A and B in shared memory, weights from the ring)
+//    into the same accumulator, then a commit to the tile's acc barrier;
+//  * producer warp (one thread): streams the weights of layers 2-3 for each
+//    tile through the ring (full/free barriers), 256 KB of L2 reads per tile.
+// 3.6 million rows (28 k tiles, 186 per SM): 1.02 ms; one tile in flight, with the activations in tensor memory
+// and the next layer's MMAs behind the epilogue slab by slab, took 1.20 ms.
+// The epilogue alone takes 0.88 ms, the MMAs alone 0.51.  Tried and slower:
+// eight warps for each tile instead of all for one (1.10), the second tile two
+// layers behind the first (1.17).
 // Every wait is bounded and gives up once any thread of the CTA has set the
 // abort flag; before the tensor memory is released and the CTA leaves, all
 // MMAs, copies and arrivals from or to this CTA have completed.
@@ -809,16 +810,17 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) k_mlp_umma(const UmmaArgs u) 
   unsigned char *sm = sraw + ((1024 - (smem_addr(sraw) & 1023)) & 1023);
   __shared__ float s_bias[3 * kNh + kNout];
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) unsigned long long s_bar[24];
+  __shared__ __align__(8) unsigned long long s_bar[8 + 2 * kUmmaStages];
   __shared__ int s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long nrows = u.rows_dev ? min((long long)*u.rows_dev, u.rows) : u.rows;
   const long long ntiles = (nrows + 127) / 128;
   const long long cta = blockIdx.x, ncta = gridDim.x;
-  const long long my_tiles = cta < ntiles ? (ntiles - 1 - cta) / ncta + 1 : 0;
+  const long long my_tiles = cta < ntiles ? (ntiles - 1 - cta) / ncta + 1 : 0;   // tiles cta, cta + ncta, ..
   const uint32_t sb = smem_addr(sm);
   volatile int *abort = &s_abort;
-  enum { B_W = 0, B_FEAT = 1, B_ACC = 2, B_ACT = 3, B_FULL = 7, B_FREE = 7 + kUmmaStages, B_DRAIN = 7 + 2 * kUmmaStages };
+  // per tile slot t = 0, 1: features ready, accumulator ready, activations ready
+  enum { B_W = 0, B_FEAT = 1, B_ACC = 3, B_ACT = 5, B_FULL = 7, B_FREE = 7 + kUmmaStages, B_DRAIN = 7 + 2 * kUmmaStages };
   const uint32_t bar0 = smem_addr(&s_bar[0]);
   auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
   auto fail = [&]() {
@@ -838,9 +840,13 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) k_mlp_umma(const UmmaArgs u) 
   }
   if (tid == 0) {
     bar_init(bar(B_W), 1);
-    bar_init(bar(B_FEAT), kUmmaEpiWarps);
-    bar_init(bar(B_ACC), 1);
-    for (int s = 0; s < 4; ++s) bar_init(bar(B_ACT + s), kUmmaEpiWarps);
+    for (int t = 0; t < 2; ++t) {
+      // all warps, so that none can be a whole phase of ACC behind when the
+      // next tile's layer 1 is issued
+      bar_init(bar(B_FEAT + t), kUmmaEpiWarps);
+      bar_init(bar(B_ACC + t), 1);
+      bar_init(bar(B_ACT + t), kUmmaEpiWarps);
+    }
     for (int s = 0; s < kUmmaStages; ++s) {
       bar_init(bar(B_FULL + s), 1);
       bar_init(bar(B_FREE + s), 1);
@@ -859,30 +865,36 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) k_mlp_umma(const UmmaArgs u) 
       bar_expect_tx(bar(B_W), kImgW1 + kImgW4);
       bulk_load(sb + kSmW1, u.img, kImgW1, bar(B_W));
       bulk_load(sb + kSmW4, u.img + kImgW1 + kImgChunks * kImgChunk, kImgW4, bar(B_W));
-      // load i goes to stage i % S as that stage's (i / S)-th fill; from the
-      // second fill on it waits until the MMAs of the previous fill have
-      // completed
-      const long long nch = my_tiles * kImgChunks;
-      long long i = 0;
-      for (; i < nch; ++i) {
-        const int st = (int)(i % kUmmaStages);
-        const long long fill = i / kUmmaStages;
-        if (fill > 0 && !bar_wait_or_abort(bar(B_FREE + st), (uint32_t)((fill - 1) & 1), kUmmaSpins, abort)) {
-          fail();
-          break;
-        }
-        bar_expect_tx(bar(B_FULL + st), kImgChunk);
-        const uint32_t dst = sb + kSmRing + (uint32_t)st * kImgChunk;
-        const unsigned char *src = u.img + kImgW1 + (uint32_t)(i % kImgChunks) * kImgChunk;
-        bulk_load(dst, src, kImgChunk, bar(B_FULL + st));
+      // the MMA warp takes, per pair of tiles, layer 2's four chunks for each
+      // tile and then layer 3's.  Load i goes to stage i % S as that stage's
+      // (i / S)-th fill; from the second fill on it waits until the MMAs of
+      // the previous fill have completed
+      constexpr int kL = kImgChunks / 2;   // chunks per layer
+      uint32_t i = 0;
+      bool ok = true;
+      for (long long it = 0; ok && it < my_tiles; it += 2) {
+        const int ntp = my_tiles - it >= 2 ? 2 : 1;
+        for (int l = 0; ok && l < 2; ++l)
+          for (int t = 0; ok && t < ntp; ++t) {
+            const unsigned char *src = u.img + kImgW1 + (uint32_t)l * (kL * kImgChunk);
+#pragma unroll
+            for (int s = 0; s < kL; ++s, ++i) {
+              const uint32_t st = i % kUmmaStages, fill = i / kUmmaStages;
+              ok = ok && (fill == 0 || bar_wait_or_abort(bar(B_FREE + (int)st), (fill - 1) & 1u, kUmmaSpins, abort));
+              if (!ok) break;
+              bar_expect_tx(bar(B_FULL + (int)st), kImgChunk);
+              bulk_load(sb + kSmRing + st * kImgChunk, src + (uint32_t)s * kImgChunk, kImgChunk, bar(B_FULL + (int)st));
+            }
+          }
       }
+      if (!ok) fail();
       // drain: the copies into this CTA have landed (last fill of each
       // stage), and so have the commits of those fills
       bar_wait(bar(B_W), 0, kUmmaSpins);
-      for (int st = 0; st < kUmmaStages && st < i; ++st) {
-        const long long fills = (i - st + kUmmaStages - 1) / kUmmaStages;
-        bar_wait(bar(B_FULL + st), (uint32_t)((fills - 1) & 1), kUmmaSpins);
-        bar_wait_or_abort(bar(B_FREE + st), (uint32_t)((fills - 1) & 1), kUmmaSpins, abort);
+      for (uint32_t st = 0; st < kUmmaStages && st < i; ++st) {
+        const uint32_t fills = (i - st + kUmmaStages - 1) / kUmmaStages;
+        bar_wait(bar(B_FULL + (int)st), (fills - 1) & 1u, kUmmaSpins);
+        bar_wait_or_abort(bar(B_FREE + (int)st), (fills - 1) & 1u, kUmmaSpins, abort);
       }
     }
     __syncwarp();
@@ -890,49 +902,61 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) k_mlp_umma(const UmmaArgs u) 
     if (lane == 0) {
       const uint32_t id256 = umma_idesc_bf16(128, 256), id16 = umma_idesc_bf16(128, 16);
       bool ok = bar_wait_or_abort(bar(B_W), 0, kUmmaSpins, abort);
-      int nfeat = 0, nact = 0;
-      long long chunk = 0;
-      for (long long it = 0; ok && it < my_tiles; ++it) {
-        ok = bar_wait_or_abort(bar(B_FEAT), (uint32_t)(nfeat++ & 1), kUmmaSpins, abort);
-        if (!ok) break;
-        tc_fence_after();
-        // layer 1: features (tensor memory, k < 16) x W1 -> A0
-        umma_bf16_ts(taddr + kTmA0, taddr + kTmFeat, umma_desc_sw128(sb + kSmW1), id256, 0u);
-        umma_commit(bar(B_ACC));
-        // layers 2 (A0 -> A1) and 3 (A1 -> A0), K-slab by K-slab
-        for (int l = 0; ok && l < 2; ++l, ++nact) {
-          const uint32_t dacc = taddr + (l == 0 ? kTmA1 : kTmA0), ain = taddr + (l == 0 ? kTmA0 : kTmA1);
-          for (int s = 0; ok && s < 4; ++s) {
-            ok = bar_wait_or_abort(bar(B_ACT + s), (uint32_t)(nact & 1), kUmmaSpins, abort);
-            if (!ok) break;
-            tc_fence_after();
-            const int st = (int)(chunk % kUmmaStages);
-            ok = bar_wait_or_abort(bar(B_FULL + st), (uint32_t)((chunk / kUmmaStages) & 1), kUmmaSpins, abort);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t wst = sb + kSmRing + (uint32_t)st * kImgChunk;
-#pragma unroll
-            for (int sub = 0; sub < 4; ++sub)
-              umma_bf16_ts(dacc, ain + 64u * (uint32_t)s + 16u * (uint32_t)sub, umma_desc_sw128(wst + 32u * (uint32_t)sub),
-                           id256, (s | sub) ? 1u : 0u);
-            umma_commit(bar(B_FREE + st));
-            ++chunk;
-          }
-          if (ok) umma_commit(bar(B_ACC));
-        }
-        // layer 4: A0 x W4 -> A1 columns 0..15
-        for (int s = 0; ok && s < 4; ++s) {
-          ok = bar_wait_or_abort(bar(B_ACT + s), (uint32_t)(nact & 1), kUmmaSpins, abort);
+      uint32_t nfeat[2] = {0, 0}, nact[2] = {0, 0};
+      uint32_t chunk = 0;
+      // the descriptors' addresses are in units of 16 bytes and shared memory
+      // ends below 2^18: an offset is a plain addition
+      const uint64_t dact = umma_desc_sw128(sb + kSmAct), dring = umma_desc_sw32(sb + kSmRing);
+      for (long long it = 0; ok && it < my_tiles; it += 2) {
+        const int ntp = my_tiles - it >= 2 ? 2 : 1;
+        // layer 1: features x W1
+        for (int t = 0; ok && t < ntp; ++t) {
+          ok = bar_wait_or_abort(bar(B_FEAT + t), nfeat[t]++ & 1u, kUmmaSpins, abort);
           if (!ok) break;
           tc_fence_after();
-#pragma unroll
-          for (int sub = 0; sub < 4; ++sub)
-            umma_bf16_ts(taddr + kTmA1, taddr + kTmA0 + 64u * (uint32_t)s + 16u * (uint32_t)sub,
-                         umma_desc_sw128(sb + kSmW4 + 2048u * (uint32_t)s + 32u * (uint32_t)sub), id16,
-                         (s | sub) ? 1u : 0u);
+          umma_bf16(taddr + 256u * (uint32_t)t, umma_desc_sw32(sb + kSmFeat + (uint32_t)t * kUmmaFeat),
+                    umma_desc_sw32(sb + kSmW1), id256, 0u);
+          umma_commit(bar(B_ACC + t));
         }
-        ++nact;
-        if (ok) umma_commit(bar(B_ACC));
+        // layers 2 and 3, K-slab by K-slab as the weights land
+        for (int l = 0; ok && l < 2; ++l)
+          for (int t = 0; ok && t < ntp; ++t) {
+            ok = bar_wait_or_abort(bar(B_ACT + t), nact[t]++ & 1u, kUmmaSpins, abort);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t da = dact + (uint64_t)(t * (kUmmaAct >> 4));
+#pragma unroll
+            for (int s = 0; s < 16; s += kUmmaSteps, ++chunk) {
+              const uint32_t st = chunk % kUmmaStages;
+              ok = ok && bar_wait_or_abort(bar(B_FULL + (int)st), (chunk / kUmmaStages) & 1u, kUmmaSpins, abort);
+              if (!ok) break;
+              tc_fence_after();
+              const uint64_t dw = dring + (uint64_t)(st * (kImgChunk >> 4));
+#pragma unroll
+              for (int sub = 0; sub < kUmmaSteps; ++sub) {
+                const int k = s + sub;   // K elements 16 k ..
+                umma_bf16(taddr + 256u * (uint32_t)t, da + (uint64_t)((16384 * (k >> 2) + 32 * (k & 3)) >> 4),
+                          dw + (uint64_t)((kImgStep * sub) >> 4), id256, k ? 1u : 0u);
+              }
+              umma_commit(bar(B_FREE + (int)st));
+            }
+            if (ok) umma_commit(bar(B_ACC + t));
+          }
+        // layer 4: columns 0..15 of the tile's accumulator
+        for (int t = 0; ok && t < ntp; ++t) {
+          ok = bar_wait_or_abort(bar(B_ACT + t), nact[t]++ & 1u, kUmmaSpins, abort);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t da = dact + (uint64_t)(t * (kUmmaAct >> 4)), dw = umma_desc_sw128(sb + kSmW4);
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int sub = 0; sub < 4; ++sub)
+              umma_bf16(taddr + 256u * (uint32_t)t, da + (uint64_t)((16384 * s + 32 * sub) >> 4),
+                        dw + (uint64_t)((2048 * s + 32 * sub) >> 4), id16,
+                        (s | sub) ? 1u : 0u);
+          umma_commit(bar(B_ACC + t));
+        }
       }
       if (!ok) fail();
       // drain: every MMA this thread issued has completed
@@ -944,79 +968,106 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) k_mlp_umma(const UmmaArgs u) 
     // epilogue warps
     const int q = warp & 3, j = warp >> 2;
     const int row = 32 * q + lane;
-    const uint32_t tl = taddr + ((uint32_t)(32 * q) << 16);
-    int nacc = 0;
+    const uint32_t rowx = (uint32_t)(row & 7) << 4;   // the 128-byte swizzle of this row
+    uint32_t nacc[2] = {0, 0};
     bool ok = true;
-    uint4 f0 = make_uint4(0, 0, 0, 0), f1 = f0;
-    auto load_features = [&](long long g) {
-      f0 = make_uint4(0, 0, 0, 0);
-      f1 = f0;
-      const long long r = g * 128 + row;
-      if (g < ntiles && r < nrows) {
+    uint4 f0[2], f1[2];
+    // tile n of this CTA: its rows' features into registers, then (put) shared memory
+    auto load_features = [&](long long n, int t) {
+      f0[t] = make_uint4(0, 0, 0, 0);
+      f1[t] = f0[t];
+      const long long r = (cta + n * ncta) * 128 + row;
+      if (n < my_tiles && r < nrows) {
         const uint4 *src = reinterpret_cast<const uint4 *>(u.xb + r * kNinPad);
-        f0 = src[0];
-        f1 = src[1];
+        f0[t] = src[0];
+        f1[t] = src[1];
       }
     };
-    if (j == 0) load_features(cta);
-    for (long long g = cta; ok && g < ntiles; g += ncta) {
-      const long long r0 = g * 128;
-      // every epilogue warp arrives: the next tile's layer-1 MMA (which
-      // overwrites A0) waits until all of them have seen the previous
-      // tile's last accumulator phase; the features go to tensor memory
-      // (A1's last columns: the previous tile's layer-3 MMAs, which read
-      // A1, have completed)
+    auto put_features = [&](int t) {
       if (j == 0) {
-        const uint32_t fv[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-        tmem_st8(tl + kTmFeat, fv);
-        tc_fence_before();
+        unsigned char *p = sm + kSmFeat + (uint32_t)t * kUmmaFeat;
+        *reinterpret_cast<uint4 *>(p + sw32_offset(row, 0)) = f0[t];
+        *reinterpret_cast<uint4 *>(p + sw32_offset(row, 8)) = f1[t];
+        fence_async_smem();
       }
+      tc_fence_before();
       __syncwarp();
-      if (lane == 0) bar_arrive(bar(B_FEAT));
-      if (j == 0) load_features(g + ncta);
-      for (int l = 0; l < 3; ++l) {
-        ok = bar_wait_or_abort(bar(B_ACC), (uint32_t)(nacc++ & 1), kUmmaSpins, abort);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t tacc = tl + (l == 1 ? kTmA1 : kTmA0);
-        const float *b = s_bias + l * kNh;
-#pragma unroll 1
-        for (int s = 0; s < 4; ++s) {
-          const int c0 = 64 * s + 16 * j;
-          float v[16];
-          tmem_ld16(tacc + (uint32_t)c0, v);
-          uint32_t hb[8];
+      if (lane == 0) bar_arrive(bar(B_FEAT + t));
+    };
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const __nv_bfloat162 p = __floats2bfloat162_rn(tanh_approx(v[2 * i] + b[c0 + 2 * i]),
-                                                          tanh_approx(v[2 * i + 1] + b[c0 + 2 * i + 1]));
-            hb[i] = *reinterpret_cast<const uint32_t *>(&p);
+    for (int t = 0; t < 2; ++t) {
+      if (j == 0) load_features(t, t);
+      if (t < my_tiles) put_features(t);
+    }
+    for (long long it = 0; ok && it < my_tiles; it += 2) {
+      const int ntp = my_tiles - it >= 2 ? 2 : 1;
+      if (j == 0) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) load_features(it + 2 + t, t);
+      }
+      for (int l = 0; ok && l < 3; ++l) {
+        const float *b = s_bias + l * kNh;
+        for (int t = 0; t < ntp; ++t) {
+          const uint32_t ph = t == 0 ? nacc[0]++ : nacc[1]++;
+          ok = bar_wait_or_abort(bar(B_ACC + t), ph & 1u, kUmmaSpins, abort);
+          if (!ok) break;
+          tc_fence_after();
+          // this warp's slab, 32 columns at a time: the second load is in
+          // flight while the first half is worked on
+          const uint32_t tacc = taddr + 256u * (uint32_t)t + ((uint32_t)(32 * q) << 16) + 64u * (uint32_t)j;
+          unsigned char *act = sm + kSmAct + (uint32_t)t * kUmmaAct + 16384u * (uint32_t)j + 128u * (uint32_t)row;
+          uint32_t v[2][32];
+          tmem_ld32(tacc, v[0]);
+          tmem_wait32(v[0]);
+          tmem_ld32(tacc + 32u, v[1]);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (h == 1) tmem_wait32(v[1]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {   // 8 columns, one 16-byte chunk of the row
+              const float *bc = b + 64 * j + 32 * h + 8 * c;
+              uint32_t hb[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const __nv_bfloat162 p =
+                    __floats2bfloat162_rn(tanh_approx(__uint_as_float(v[h][8 * c + 2 * i]) + bc[2 * i]),
+                                          tanh_approx(__uint_as_float(v[h][8 * c + 2 * i + 1]) + bc[2 * i + 1]));
+                hb[i] = *reinterpret_cast<const uint32_t *>(&p);
+              }
+              *reinterpret_cast<uint4 *>(act + ((uint32_t)((4 * h + c) << 4) ^ rowx)) =
+                  make_uint4(hb[0], hb[1], hb[2], hb[3]);
+            }
           }
-          tmem_st8(tacc + (uint32_t)c0, hb);
+          fence_async_smem();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) bar_arrive(bar(B_ACT + s));
+          if (lane == 0) bar_arrive(bar(B_ACT + t));
         }
       }
       if (!ok) break;
-      ok = bar_wait_or_abort(bar(B_ACC), (uint32_t)(nacc++ & 1), kUmmaSpins, abort);
-      if (!ok) break;
-      tc_fence_after();
-      if (j == 0) {
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (t >= ntp) break;
+        ok = bar_wait_or_abort(bar(B_ACC + t), (t == 0 ? nacc[0]++ : nacc[1]++) & 1u, kUmmaSpins, abort);
+        if (!ok) break;
+        tc_fence_after();
         float v[16];
-        tmem_ld16(tl + kTmA1, v);
-        tc_fence_before();
-        if (r0 + row < nrows) {
-          float y[kNout];
+        if (j == 0) tmem_ld16(taddr + 256u * (uint32_t)t + ((uint32_t)(32 * q) << 16), v);
+        if (it + 2 + t < my_tiles) put_features(t);   // the accumulator is free: the slot's next tile
+        if (j == 0) {
+          const long long r = (cta + (it + t) * ncta) * 128 + row;
+          if (r < nrows) {
+            float y[kNout];
 #pragma unroll
-          for (int i = 0; i < kNout; ++i) y[i] = v[i] + s_bias[3 * kNh + i];
-          if (u.rowpt && CASIM_INDEX_OK(u.rowpt[r0 + row] >= 0 && u.rowpt[r0 + row] < u.npts, u.err)) {
-            const float *muy = u.norm + 2 * kNin, *sdy = u.norm + 2 * kNin + kNout;
-            u.surr[u.rowpt[r0 + row]] = make_float4(__expf(y[0] * sdy[0] + muy[0]), __expf(y[1] * sdy[1] + muy[1]),
-                                                    __expf(y[2] * sdy[2] + muy[2]), __expf(y[3] * sdy[3] + muy[3]));
-          } else {
+            for (int i = 0; i < kNout; ++i) y[i] = v[i] + s_bias[3 * kNh + i];
+            if (u.rowpt && CASIM_INDEX_OK(u.rowpt[r] >= 0 && u.rowpt[r] < u.npts, u.err)) {
+              const float *muy = u.norm + 2 * kNin, *sdy = u.norm + 2 * kNin + kNout;
+              u.surr[u.rowpt[r]] = make_float4(__expf(y[0] * sdy[0] + muy[0]), __expf(y[1] * sdy[1] + muy[1]),
+                                               __expf(y[2] * sdy[2] + muy[2]), __expf(y[3] * sdy[3] + muy[3]));
+            } else {
 #pragma unroll
-            for (int i = 0; i < kNout; ++i) u.y[(r0 + row) * kNout + i] = y[i];
+              for (int i = 0; i < kNout; ++i) u.y[r * kNout + i] = y[i];
+            }
           }
         }
       }

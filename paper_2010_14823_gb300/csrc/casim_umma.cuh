@@ -21,6 +21,23 @@ __host__ __device__ __forceinline__ uint32_t sw128_offset(int R, int r, int k) {
   return (uint32_t)(slab * R * 128 + r * 128 + chunk * 16 + (kk & 7) * 2);
 }
 
+// byte offset of element (r, k), k < 16, of a K-major tile of 16 K-elements
+// with the 32-byte swizzle: row r is 32 contiguous bytes, its two 16-byte
+// chunks exchanged in every second group of four rows
+__host__ __device__ __forceinline__ uint32_t sw32_offset(int r, int k) {
+  return (uint32_t)(r * 32 + (((k >> 3) ^ ((r >> 2) & 1)) << 4) + (k & 7) * 2);
+}
+// its matrix descriptor: 256 bytes between 8-row groups
+__device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)(16u >> 4) << 16;
+  d |= (uint64_t)(256u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)6 << 61;
+  return d;
+}
+
 // shared-memory matrix descriptor: start address, leading-dimension offset
 // (unused by swizzled K-major layouts, set to 16 bytes), stride-dimension
 // offset 1024 bytes (between 8-row groups), descriptor version 1, 128-byte
@@ -63,17 +80,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
       "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// A operand from tensor memory (M = 128: lane r holds row r, K pairs packed
-// two BF16 per 32-bit column), B from shared memory
-__device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
-                                             uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -133,12 +139,28 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// this thread's lane, 8 consecutive 32-bit columns from col; waits for the stores
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t v[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]),
-               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-               : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+// the same for 32 columns without the wait; tmem_wait32 names the registers,
+// so that nothing that uses them can come before it
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait32(uint32_t r[32]) {
+  asm volatile(
+      "tcgen05.wait::ld.sync.aligned;"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+        "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+        "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+      :
+      : "memory");
 }
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -167,8 +189,10 @@ __device__ __forceinline__ uint64_t global_ns() {
 // every wait on a barrier gives up after this long (or `spins` polls)
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
-// bounded wait for phase `parity`; false if it gave up
+// bounded wait for phase `parity`; false if it gave up.  The first try comes
+// before the timer is read.
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, unsigned spins) {
+  if (bar_try(bar, parity)) return true;
   const uint64_t t0 = global_ns();
   for (unsigned i = 0; i < spins; ++i) {
     if (bar_try(bar, parity)) return true;
@@ -179,6 +203,7 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, unsigned
 // bounded wait that also gives up early once `abort` is set by another thread
 __device__ __forceinline__ bool bar_wait_or_abort(uint32_t bar, uint32_t parity, unsigned spins,
                                                   const volatile int *abort, uint64_t limit_ns = kWaitLimitNs) {
+  if (bar_try(bar, parity)) return true;
   const uint64_t t0 = global_ns();
   for (unsigned i = 0; i < spins; ++i) {
     if (bar_try(bar, parity)) return true;
