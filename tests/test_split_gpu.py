@@ -61,3 +61,19 @@ def test_split_step_equals_one_thread_per_column(flags, precision):
             b = _step(wide, dz, WIDE, flags, precision, dt, tend)
             for x, y in zip(a, b):
                 assert np.array_equal(x, y[..., :ncols]), (ncols, nlev, dt, tend)
+
+
+@pytest.mark.parametrize("flags", list(FLAGS))
+def test_blocks_of_64_threads_equal_blocks_of_128(flags):
+    """One thread per column in at most one resident wave: blocks of half the size, same bits."""
+    nlev = 13
+    dz = synth.dz_stretched(nlev)
+    base = _fields(FLAGS[flags], 700, nlev, dz, seed=31)
+    wide = np.ascontiguousarray(np.tile(base, (1, 1, -(-WIDE // 700)))[:, :, :WIDE])
+    for dt, tend in ((1.0, False), (30.0, False), (1.0, True), (30.0, True)):
+        b = _step(wide, dz, WIDE, flags, casim.CASIM_MIXED, dt, tend)
+        for ncols in (50_001, 65_536):
+            fld = np.ascontiguousarray(wide[:, :, :-(-ncols // 32) * 32])
+            a = _step(fld, dz, ncols, flags, casim.CASIM_MIXED, dt, tend)
+            for x, y in zip(a, b):
+                assert np.array_equal(x, y[..., :ncols]), (ncols, dt, tend)
