@@ -1397,8 +1397,7 @@ using Mix = MixT<PolicyMix>;
 // ice process runs and only rain sediments.
 struct PolicyF64Warm : PolicyF64 {
   static constexpr bool kWarm = true;
-  // measured on 512x512x150 stratus: 4 / 5 / 6 -> 52.3-54.3 / 49.0 / 50.4 ms per step (96
-  // registers and no spills at 5, also in the aerosol and triple-moment warm forms)
+  // measured on 512x512x150 stratus: 4 / 5 / 6 / 8 -> 7.90 / 7.93 / 7.98 / 8.05 ms per step
   static constexpr int kMinBlocks = 5;
 };
 struct PolicyMixWarm : PolicyMix {
@@ -2069,16 +2068,22 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
     float qpost[4], npost[4];
     if (act) {
       MixT<M>::template process<kTend>(K, s, a.dt, w, es0, qs0, o, a.surr ? a.surr + (size_t)k * a.pitch + c : nullptr);
-      if constexpr (!M::kWarm && !M::kAero && !M::kTri) {
+      if constexpr (!M::kWarm && !(M::kAero && kTend)) {
         // the FP64 values the increments are added to, read again from this
         // level's stage slots (they stay there until the level after next is
         // prefetched) rather than held in registers through the processes:
-        // no spills, 2.02 -> 1.95 ms per 512x512x150 step, results unchanged
+        // no spills, 2.02 -> 1.95 ms per 512x512x150 step, results unchanged;
+        // triple-moment 65 536 x 100 849 -> 836 us, 262 144 x 100 3.01 -> 2.97
+        // ms (its sixth moments too: without them 20 000 x 100 spills, 446
+        // instead of 418 us); aerosol 20 000 x 100 288 -> 277 us, 262 144 x
+        // 100 2.11 -> 2.09 ms, but its source terms 1214 -> 1230 us
         const volatile double *v = cur;
         s.T = v[0 * ss]; s.qv = v[1 * ss]; s.qc = v[2 * ss]; s.qr = v[3 * ss];
         s.qi = v[4 * ss]; s.qs = v[5 * ss]; s.qg = v[6 * ss];
         s.nc = v[7 * ss]; s.nr = v[8 * ss]; s.ni = v[9 * ss]; s.ns = v[10 * ss];
         s.ng = v[11 * ss]; s.na = v[12 * ss]; s.rho = v[14 * ss];
+#pragma unroll
+        for (int x = 0; x < nz3<M>(); ++x) zref(s, x) = v[(16 + x) * ss];
       }
       MixT<M>::apply_masses(s, o, macc);
       if constexpr (M::kTri) keep3 = MixT<M>::apply_z(K, s, w, o);
