@@ -33,24 +33,26 @@ WORKLOAD = "deep_512x512x150"
 
 # DRAM traffic of k_step<PolicyMix> on the deep-convection state, from one
 # single-pass ncu capture of the full 262 144-column x 150-level launch
-# (dram__bytes_read.sum + dram__bytes_write.sum = 5.0588 + 3.9828 GB for
+# (dram__bytes_read.sum + dram__bytes_write.sum = 5.0611 + 3.9698 GB for
 # 39.32 M points); at another column count it is scaled per point (reads are
 # 16 fields per point and writes follow the changed points).  Valid only for
 # the kernel source it was taken on.
-MEASURED_TRAFFIC = {"kernel": "k_step<PolicyMix>", "bytes_per_launch": 9041585152, "points": 39321600,
-                    "bytes_per_point": 229.94,
+MEASURED_TRAFFIC = {"kernel": "k_step<PolicyMix>", "bytes_per_launch": 9030921216, "points": 39321600,
+                    "bytes_per_point": 229.67,
                     "source": "paper_2010_14823_gb300/csrc/casim_device.cuh",
-                    "sha256": "b040dec6cc7b6d47b6f675add1fcc1f4f5979e38b72bbe9ddb8b957d05c32d1c"}
+                    "sha256": "175716eac5f3a50d281cf54ff1afe3d8df0760f9d5e3726c1ab97780908559db"}
 
 
 # FP64 arithmetic instructions of k_step<PolicyF64> per point on the same
 # state, from one ncu capture of a 16 384-column x 150-level launch
 # (smsp__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum =
-# 1168.3 M + 296.4 M + 381.0 M for 2.458 M points); the FP64 pipe was 72.9 %
+# 582.3 M + 210.9 M + 289.5 M for 2.458 M points); the FP64 pipe was 79.3 %
 # busy.  Valid only for the kernel source it was taken on.
-MEASURED_FP64_OPS = {"kernel": "k_step<PolicyF64>", "inst_per_point": 751.07,
-                     "dfma": 475.40, "dadd": 120.63, "dmul": 155.04, "fp64_pipe_active": 0.729,
-                     "sha256": "b040dec6cc7b6d47b6f675add1fcc1f4f5979e38b72bbe9ddb8b957d05c32d1c"}
+MEASURED_FP64_OPS = {"kernel": "k_step<PolicyF64>", "inst_per_point": 440.53,
+                     "dfma": 236.92, "dadd": 85.81, "dmul": 117.80, "fp64_pipe_active": 0.793,
+                     "with": {"casim_f64.cuh": "b622fbabc865a116ec75f857d71932b9070e16deec92f520d2cbf81df5cdf9bb",
+                              "casim_math64.cuh": "77319d4ef15b9df62adbc456dce9219359100983f498f8e1132fc06f027ec9dd"},
+                     "sha256": "175716eac5f3a50d281cf54ff1afe3d8df0760f9d5e3726c1ab97780908559db"}
 
 
 def _host_link_gbs(torch, stream, nbytes: int = 1 << 30):
@@ -94,9 +96,9 @@ def _host_link_gbs(torch, stream, nbytes: int = 1 << 30):
     return r
 
 
-def _kernel_source_sha() -> str:
+def _kernel_source_sha(name: str = "casim_device.cuh") -> str:
     import hashlib
-    path = os.path.join(os.path.dirname(os.path.abspath(__file__)), MEASURED_TRAFFIC["source"])
+    path = os.path.join(os.path.dirname(os.path.abspath(__file__)), os.path.dirname(MEASURED_TRAFFIC["source"]), name)
     with open(path, "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()
 
@@ -115,6 +117,8 @@ def _fp64_roofline(npts: int, fp_ms: float):
     instructions per second over the DFMA rate measured now (probe of
     include/casim_peaks.h); None if the kernel source changed since the count."""
     if _kernel_source_sha() != MEASURED_FP64_OPS["sha256"]:
+        return None
+    if any(_kernel_source_sha(f) != sha for f, sha in MEASURED_FP64_OPS["with"].items()):
         return None
     from paper_2010_14823_gb300 import peaks
     peak = peaks.peak_rate("dfma", 1 << 12)
