@@ -1205,8 +1205,6 @@ static int mlp_batch_ws(casim_mlp *m, int n) {
   if (e == cudaSuccess) e = dalloc(&m->Xn, (size_t)n * kNin);
   if (e == cudaSuccess) e = dalloc(&m->Tn, (size_t)n * kNout);
   if (e == cudaSuccess) e = dalloc(&m->Mb, (size_t)n * kNout);
-  // (columns 4.. of the output layer's BF16 gradient stay zero)
-  if (e == cudaSuccess) e = cudaMemset(m->dzb4, 0, (size_t)n * kNoutPad * sizeof(__nv_bfloat16));
   if (e != cudaSuccess) {
     mlp_free_batch(m);
     return e == cudaErrorMemoryAllocation ? CASIM_ERR_OOM : cuda_fail(e, "cudaMalloc");

@@ -148,7 +148,9 @@ struct EpiOut {
 };
 
 // masked squared error of one output: the gradient to dz (FP32 [n][4] and BF16
-// [n][16], whose columns 4.. stay zero), the loss term returned
+// [n][16]), the loss term returned.  Columns 4.. of the BF16 copy meet the zero
+// columns of w4k in the data gradient; the kernels that write a row write them
+// as zeros too, on the stream that reads them.
 __device__ __forceinline__ double mlp_loss_term(float y, float t, float m, float cnt, float &g) {
   const float inv = 1.f / fmaxf(cnt, 1.f);
   const float d = (y - t) * m;
@@ -179,9 +181,9 @@ struct EpiOutLoss {
     reinterpret_cast<float4 *>(dz)[m] = make_float4(g[0], g[1], g[2], g[3]);
     __nv_bfloat162 lo, hi;
     lo.x = h[0]; lo.y = h[1]; hi.x = h[2]; hi.y = h[3];
-    __nv_bfloat162 *d = reinterpret_cast<__nv_bfloat162 *>(dzb + (long long)m * kNoutPad);
-    d[0] = lo;
-    d[1] = hi;
+    uint4 *d = reinterpret_cast<uint4 *>(dzb + (long long)m * kNoutPad);   // 32 bytes a row
+    d[0] = make_uint4(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi), 0u, 0u);
+    d[1] = make_uint4(0u, 0u, 0u, 0u);
     return part;
   }
 };
@@ -274,7 +276,10 @@ __global__ void k_mlp_loss(const float *Y, const float *T, const float *Mk, int 
     float g;
     part = mlp_loss_term(Y[i], T[i], Mk[i], *cnt, g);
     dz[i] = g;
-    dzb[i / kNout * kNoutPad + i % kNout] = __float2bfloat16(g);
+    __nv_bfloat16 *row = dzb + i / kNout * kNoutPad + i % kNout;
+    row[0] = __float2bfloat16(g);
+#pragma unroll
+    for (int j = kNout; j < kNoutPad; j += kNout) row[j] = __float2bfloat16(0.f);
   }
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if ((threadIdx.x & 31) == 0 && part != 0.0) atomicAdd(loss, part);
