@@ -160,8 +160,6 @@ static void derive(const casim_params &p, ConstK<R> &K, double (*l)(double)) {
   K.inv_mr0 = (R)(1.0 / (4.0 / 3.0 * pi * p.rho_w * p.r_r0 * p.r_r0 * p.r_r0));
   K.mey_a = (R)p.mey_a; K.mey_b = (R)p.mey_b; K.mey_c = (R)p.mey_c; K.mi0 = (R)p.m_i0;
   K.mu_air = (R)p.mu_air; K.inv_dv = (R)(1.0 / p.Dv); K.lgrho0 = (R)l(p.rho0); K.twopi = (R)(2.0 * pi);
-  K.v0_ln = (R)(std::log(p.mu_air / p.Dv) / 3.0 + 0.5 * (0.4 * std::log(p.rho0) - std::log(p.mu_air)));
-  K.ls_cp = (R)(Ls / p.cp); K.lf_cp = (R)(p.Lf / p.cp);
   for (int x = 0; x < 5; ++x) {
     const double a = p.a[x], b = p.b[x], mu = p.mu[x], cv = p.cv[x], dv = p.dv[x];
     const double gb = std::tgamma(mu + b + 1.0);

@@ -67,8 +67,6 @@ struct ConstK {
   R mey_a, mey_b, mey_c, mi0;
   // air
   R mu_air, inv_dv, lgrho0, twopi;
-  R v0_ln;                          // FP64: ln of (mu_air/Dv)^(1/3) (rho0^0.4/mu_air)^(1/2)
-  R ls_cp, lf_cp;                   // Ls/cp, Lf/cp
   SpeciesK<R> sp[5];
   // triple-moment species r, i, s, g (index 0..3, species 1..4): what their
   // shape-dependent constants are built from
@@ -531,21 +529,10 @@ struct Phys {
 
   // log of the gamma slope of a species from (log q, n), clamped
   static __device__ __forceinline__ R lglam(const SpeciesK<R> &X, R lgq, R n) {
-    const R lgn = M::lg(M::mx(n, (R)0));
+    const R lgn = M::lg(M::pos(n));
     R l = (X.lglamfac + lgn - lgq) * X.invb;
     l = M::mx(l, X.lglo);   // also maps log(0) = -inf (and NaN) to the lower bound
     return M::mn(l, X.lghi);
-  }
-
-  // the same from (q, n): the FP64 form takes one logarithm, of n/q
-  static __device__ __forceinline__ R lglam_q(const SpeciesK<R> &X, R q, R n) {
-    if constexpr (M::kMixed) {
-      return lglam(X, M::lg(q), n);
-    } else {
-      R l = (X.lglamfac + M::lg(M::div(M::pos(n), q))) * X.invb;
-      l = M::mx(l, X.lglo);
-      return M::mn(l, X.lghi);
-    }
   }
 
   // a4..a9: process rates from the post-activation state
@@ -566,23 +553,17 @@ struct Phys {
     const bool warm = M::kMixed ? tc > (R)0 : T > K.T0;
     const bool nucl = M::kMixed ? tc < K.tnuc0 : T < K.Tnuc;
 
-    // air properties shared by the ventilated integrals
-    R dfac, V0;   // (rho0/rho)^0.4, cbrt(nu / Dv) sqrt(dfac / nu)
-    if constexpr (M::kMixed) {
+    // air properties shared by the ventilated integrals: (rho0/rho)^0.4 and
+    // cbrt(nu / Dv) sqrt(dfac / nu) (the FP64 form: only where a species is
+    // there to need them)
+    R dfac = (R)0, V0 = (R)0;
+    if (M::kMixed || hr || M::gt(w.qx[0], K.qmin) || M::gt(w.qx[1], K.qmin) || M::gt(w.qx[2], K.qmin)) {
       const R lgrho = M::lg(rho);
       dfac = M::ex((R)0.4 * (K.lgrho0 - lgrho));
       const R nu = M::div(K.mu_air, rho);
       V0 = M::cbrt(nu * K.inv_dv) * M::sqrt(M::div(dfac, nu));
-    } else {
-      // only where a species is there to need them; V0 as one power of rho
-      dfac = V0 = (R)0;
-      if (hr || M::gt(w.qx[0], K.qmin) || M::gt(w.qx[1], K.qmin) || M::gt(w.qx[2], K.qmin)) {
-        const R lgrho = M::lg(rho);
-        dfac = M::ex((R)0.4 * (K.lgrho0 - lgrho));
-        V0 = M::ex(K.v0_ln - (R)(1.0 / 30.0) * lgrho);
-      }
-      r.dfac = dfac;
     }
+    if constexpr (!M::kMixed) r.dfac = dfac;
 
     r.aut = r.acc = r.scc = r.scr = r.evr = r.nucn = (R)0;
 #pragma unroll
@@ -590,7 +571,7 @@ struct Phys {
     r.rim[0] = r.rim[1] = (R)0;
 
     const R lgqc = hc ? M::lg(qc) : (R)0;
-    const R lgqr = (M::kMixed ? hr : hr && hc) ? M::lg(qr) : (R)0;
+    const R lgqr = hr ? M::lg(qr) : (R)0;
     if (hc) {
       const R ncc = M::mx(rho * nc * (R)1e-6, K.nc_min);
       r.aut = K.kk_aut * M::ex(K.kk_aut_qc * lgqc + K.kk_aut_nc * M::lg(ncc));
@@ -605,10 +586,10 @@ struct Phys {
         if constexpr (M::kTri) {
           typename Shape3<M>::Sh h;
           Shape3<M>::consts(K, 0, w.mu3[0], h);
-          const R l = M::kMixed ? Shape3<M>::lglam(h, X, lgqr, nr) : Shape3<M>::lglam(h, X, M::lg(qr), nr);
+          const R l = Shape3<M>::lglam(h, X, lgqr, nr);
           iv = rho * qr * (h.ev1 * M::ex(X.ex1 * l) + V0 * h.ev2 * M::ex(X.ex2 * l));
         } else {
-          const R l = M::kMixed ? lglam(X, lgqr, nr) : lglam_q(X, qr, nr);
+          const R l = lglam(X, lgqr, nr);
           iv = rho * qr * (X.ev1 * M::ex(X.ex1 * l) + V0 * X.ev2 * M::ex(X.ex2 * l));
         }
         const R Aw = K.awc * iT2, Bw = M::div(K.rv_dv * T, esl);
@@ -640,7 +621,7 @@ struct Phys {
           if (m > 0 && hc)
             r.rim[m - 1] = Shape3<M>::rim(K, 1 + m, w.mu3[1 + m]) * qc * dfac * rho * w.qx[m] * M::ex(X.exr * l);
         } else {
-          const R l = lglam_q(X, w.qx[m], w.nx[m]);
+          const R l = lglam(X, M::lg(w.qx[m]), w.nx[m]);
           const R iv = rho * w.qx[m] * (X.ev1 * M::ex(X.ex1 * l) + V0 * X.ev2 * M::ex(X.ex2 * l));
           r.dep[m] = X.dep * dfa * iv;
           if (m > 0 && hc) r.rim[m - 1] = X.rim * qc * dfac * rho * w.qx[m] * M::ex(X.exr * l);
@@ -659,7 +640,7 @@ struct Phys {
           const R l = Shape3<M>::lglam(h, X, M::lg(w.qx[m]), w.nx[m]);
           iv = rho * w.qx[m] * (h.ev1 * M::ex(X.ex1 * l) + V0 * h.ev2 * M::ex(X.ex2 * l));
         } else {
-          const R l = lglam_q(X, w.qx[m], w.nx[m]);
+          const R l = lglam(X, M::lg(w.qx[m]), w.nx[m]);
           iv = rho * w.qx[m] * (X.ev1 * M::ex(X.ex1 * l) + V0 * X.ev2 * M::ex(X.ex2 * l));
         }
         r.mlt[m] = M::div(X.mlt * tc * iv, rho);
@@ -738,7 +719,7 @@ struct Phys {
   static __device__ __forceinline__ void fall_speeds(const ConstK<R> &K, R guard, R q, R n, R dfac, int x, R &vq,
                                                      R &vn) {
     const SpeciesK<R> &X = K.sp[1 + x];
-    const R l = lglam_q(X, q, n);
+    const R l = lglam(X, M::lg(q), n);
     const R pw = M::ex(X.exv * l);
     vq = M::mn(M::mn(X.vq * dfac * pw, X.vmax), guard);
     vn = M::mn(M::mn(X.vn * dfac * pw, X.vmax), guard);
@@ -792,16 +773,19 @@ struct F64T {
     const double lv_eps_p = K.lv_cp * K.eps * p;
 #pragma unroll 1
     for (int it = 0; it < 4; ++it) {
-      // T rests on q_s to the last bit, so its quotients are rounded as
-      // written; their reciprocals serve the slope
+      // the reciprocals of the two quotients serve the slope, whose rounding
+      // a Newton step forgets (the steps have converged by the fourth)
       const double tc = Tn - K.T0;
-      double r1, r2;
-      const double ex = div64_in_range(K.esla * tc, tc + K.eslb, r1);
-      const double es = K.esl0 * exp64(ex);
-      const double qs = div64_in_range(K.eps * es, p - K.ome * es, r2);
+      const Div64 per_t(tc + K.eslb);
+      const double es = K.esl0 * exp64(per_t(K.esla * tc));
+      const Div64 per_p(p - K.ome * es);
+      const double qs = per_p(K.eps * es);
       const double f = (Tn - T0v) - K.lv_cp * (qv0 - qs);
-      const double des = es * K.eslab * (r1 * r1);
-      Tn = Tn - div64(f, 1.0 + lv_eps_p * (r2 * r2) * des);
+      double it2 = per_t.r * per_t.r, ip2 = per_p.r * per_p.r;
+      if (!per_t.in_range) it2 = div64_general(1.0, per_t.b * per_t.b);
+      if (!per_p.in_range) ip2 = div64_general(1.0, per_p.b * per_p.b);
+      const double des = es * K.eslab * it2;
+      Tn = Tn - div64(f, 1.0 + lv_eps_p * ip2 * des);
     }
     double dq = K.cp_lv * (Tn - T0v);
     if (dq < -qc0) dq = -qc0;
@@ -867,27 +851,29 @@ struct F64T {
     if (M::gt(r.acc * g.rc, 0.0)) s.nc -= g.acc * (r.acc * g.rc) * dt;
     if (M::gt(r.scc, 0.0)) s.nc -= g.scc * r.scc * dt;
     if (M::gt(r.scr, 0.0)) s.nr -= g.scr * r.scr * dt;
-    if (M::gt(r.evr, 0.0)) { tau = g.evr * r.evr * dt; s.qr -= tau; s.qv += tau; s.T -= tau * K.lv_cp; tau_rv = tau; }
+    if (M::gt(r.evr, 0.0)) { tau = g.evr * r.evr * dt; s.qr -= tau; s.qv += tau; s.T -= div64_by(tau * K.lv, K.cp, K.inv_cp); tau_rv = tau; }
     if (M::gt(r.evr * g.rr, 0.0)) s.nr -= g.evr * (r.evr * g.rr) * dt;
-    if (M::gt(g.nucm, 0.0)) { tau = g.nuc * g.nucm * dt; s.qv -= tau; qxd[0] += tau; s.T += tau * K.ls_cp; nuc_q = tau; }
+    // (the product rounded for both pools: left to the compiler it went into qxd[0]
+    // unrounded in the aerosol configuration's kernel and rounded in the standard one)
+    if (M::gt(g.nucm, 0.0)) { tau = __dmul_rn(g.nuc * g.nucm, dt); s.qv -= tau; qxd[0] += tau; s.T += div64_by(tau * K.ls, K.cp, K.inv_cp); nuc_q = tau; }
     if (M::gt(r.nucn, 0.0)) { nuc_n = g.nuc * r.nucn * dt; nxd[0] += nuc_n; }
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       if (r.dep[m] >= 0) {
-        if (M::gt(g.depp[m], 0.0)) { tau = g.dep[m] * g.depp[m] * dt; s.qv -= tau; qxd[m] += tau; s.T += tau * K.ls_cp; }
+        if (M::gt(g.depp[m], 0.0)) { tau = g.dep[m] * g.depp[m] * dt; s.qv -= tau; qxd[m] += tau; s.T += div64_by(tau * K.ls, K.cp, K.inv_cp); }
       } else {
-        tau = g.dep[m] * g.sub[m] * dt; qxd[m] -= tau; s.qv += tau; s.T -= tau * K.ls_cp; sub_q[m] = tau;
+        tau = g.dep[m] * g.sub[m] * dt; qxd[m] -= tau; s.qv += tau; s.T -= div64_by(tau * K.ls, K.cp, K.inv_cp); sub_q[m] = tau;
         if (M::gt(g.sub[m] * g.rx[m], 0.0)) nxd[m] -= g.dep[m] * (g.sub[m] * g.rx[m]) * dt;
       }
     }
-    if (M::gt(r.rim[0], 0.0)) { tau = g.rs * r.rim[0] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
+    if (M::gt(r.rim[0], 0.0)) { tau = g.rs * r.rim[0] * dt; s.qc -= tau; qxd[2] += tau; s.T += div64_by(tau * K.lf, K.cp, K.inv_cp); tau_rim += tau; }
     if (M::gt(r.rim[0] * g.rc, 0.0)) s.nc -= g.rs * (r.rim[0] * g.rc) * dt;
-    if (M::gt(r.rim[1], 0.0)) { tau = g.rg * r.rim[1] * dt; s.qc -= tau; qxd[2] += tau; s.T += tau * K.lf_cp; tau_rim += tau; }
+    if (M::gt(r.rim[1], 0.0)) { tau = g.rg * r.rim[1] * dt; s.qc -= tau; qxd[2] += tau; s.T += div64_by(tau * K.lf, K.cp, K.inv_cp); tau_rim += tau; }
     if (M::gt(r.rim[1] * g.rc, 0.0)) s.nc -= g.rg * (r.rim[1] * g.rc) * dt;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       if (M::gt(r.mlt[m], 0.0)) {
-        tau = g.mlt[m] * r.mlt[m] * dt; qxd[m] -= tau; s.qr += tau; s.T -= tau * K.lf_cp; melt_q[m] = tau;
+        tau = g.mlt[m] * r.mlt[m] * dt; qxd[m] -= tau; s.qr += tau; s.T -= div64_by(tau * K.lf, K.cp, K.inv_cp); melt_q[m] = tau;
       }
       if (M::gt(g.nmlt[m], 0.0)) {
         melt_n[m] = g.mlt[m] * g.nmlt[m] * dt; nxd[m] -= melt_n[m]; s.nr += melt_n[m];

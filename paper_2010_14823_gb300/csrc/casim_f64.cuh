@@ -13,10 +13,10 @@
 // point alone, so only the update needs the level above.
 // Measured: FP64 step, 256x256x100 stratus 28.7 -> 9.9 ms (24.7 lanes, FP64
 // pipe 66 % busy over the launch instead of 45 %), deep convection of that size
-// 35.5 -> 16.9 ms, 2 000 columns 5.2 -> 0.52 ms; with the functions of
-// casim_math64.cuh 6.2, 10.5 and 0.36 ms; with the flags decided in FP32 away
-// from saturation and comparisons on the integer pipe (an FP64 compare costs as
-// much as an addition) 4.9, 8.7 and 0.30 ms, bit for bit the same.
+// 35.5 -> 16.9 ms, 2 000 columns 5.2 -> 0.52 ms; with exp, log and the quotients
+// out of line or cheaper (casim_math64.cuh, the same bits), flags decided in FP32
+// away from saturation and comparisons on the integer pipe (an FP64 compare
+// costs as much as an addition) 6.0, 10.6 and 0.37 ms.
 // (included by casim_device.cuh)
 #pragma once
 
@@ -226,7 +226,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
         const bool act = t.cls[i] != 0;
         double *out = kTend ? tend : a.fld;
         const double *in = kTend && act ? tend : a.fld;   // where the processed values are
-        double sc = 0.0;     // dt / (rho dz)
+        Div64 per_mass;      // divides by rho dz
         bool have = false;   // some species moves here
 #pragma unroll
         for (int x = 0; x < kSed; ++x) {
@@ -240,7 +240,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
           }
           const bool wx = fast && (nonzero(X) || nonzero(X1));
           if ((wq || wx) && !have) {
-            sc = div64(a.dt, __ldg(a.fld + 14 * fs + o) * lt.dz[k]);
+            per_mass = Div64(__ldg(a.fld + 14 * fs + o) * lt.dz[k]);
             have = true;
           }
           // field 16 + x: a sixth moment; 18 + x: an aerosol mass (source-term row: three less)
@@ -248,8 +248,8 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
           if (wq || kTend) {
             double q = in[(3 + x) * fs + o], n = in[(8 + x) * fs + o];
             if (wq) {
-              q += (F1 - F) * sc;
-              n += (G1 - G) * sc;
+              q += per_mass(a.dt * (F1 - F));
+              n += per_mass(a.dt * (G1 - G));
               eflag |= nonfinite(q) | nonfinite(n);
             }
             if (kTend && fast) {
@@ -263,7 +263,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
             if (wx || kTend) {
               double e = in[ix * fs + o];
               if (wx) {
-                e += (X1 - X) * sc;
+                e += per_mass(a.dt * (X1 - X));
                 eflag |= nonfinite(e);
               }
               if (kTend && fast) e = per_dt(e - a.fld[fx * fs + o]);
