@@ -230,10 +230,23 @@ struct PolicyF64 {
   static __device__ __forceinline__ R div(R a, R b) { return div64(a, b); }
   static __device__ __forceinline__ R mn(R a, R b) { return a < b ? a : b; }
   static __device__ __forceinline__ R mx(R a, R b) { return a > b ? a : b; }
-  // a > b for a and b not both negative, on the integer pipe (an FP64 compare
-  // costs as much as an addition): IEEE values of that kind order as their bits
-  static __device__ __forceinline__ bool gt(R a, R b) { return __double_as_longlong(a) > __double_as_longlong(b); }
-  static __device__ __forceinline__ R pos(R a) { return __double2hiint(a) < 0 ? 0.0 : a; }   // max(a, 0)
+  // a > b on the integer pipe (an FP64 compare costs as much as an addition):
+  // IEEE values that are not both negative order as their bits.  NaN compares
+  // false, as in the comparison itself; gt is for a number b >= 0, gt_any for
+  // any b and a >= 0.
+  static constexpr long long kInf = 0x7ff0000000000000ll;
+  static __device__ __forceinline__ bool gt(R a, R b) {
+    const long long x = __double_as_longlong(a);
+    return x > __double_as_longlong(b) && x <= kInf;
+  }
+  static __device__ __forceinline__ bool gt_any(R a, R b) {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    // negative y: -0 equals a zero a, NaN lies above -inf
+    return x > y && x <= kInf && (y >= 0 || ((x | (y << 1)) != 0 && (unsigned long long)y <= 0xfff0000000000000ull));
+  }
+  static __device__ __forceinline__ R pos(R a) {   // max(a, 0), 0 for NaN
+    return (unsigned long long)__double_as_longlong(a) <= (unsigned long long)kInf ? a : 0.0;
+  }
 };
 
 struct PolicyMix {
@@ -276,6 +289,7 @@ struct PolicyMix {
   static __device__ __forceinline__ R mn(R a, R b) { return fminf(a, b); }
   static __device__ __forceinline__ R mx(R a, R b) { return fmaxf(a, b); }
   static __device__ __forceinline__ bool gt(R a, R b) { return a > b; }
+  static __device__ __forceinline__ bool gt_any(R a, R b) { return a > b; }
   static __device__ __forceinline__ R pos(R a) { return fmaxf(a, 0.f); }
 };
 
@@ -682,7 +696,7 @@ struct Phys {
     }
     auto fac = [&](R S, R X) -> R {
       if constexpr (!M::kMixed) {
-        return M::gt(S * dtr, X) ? M::div(M::pos(X), S * dtr) : (R)1;
+        return M::gt_any(S * dtr, X) ? M::div(M::pos(X), S * dtr) : (R)1;
       } else {
         // FP32 factor shrunk by 2^-18 so that the rounded transfers can
         // never take more than the pool holds
@@ -756,11 +770,11 @@ struct F64T {
   // 2: so, above; 3: not by adjustment
   static __device__ __forceinline__ unsigned flag(const ConstK<double> &K, const ConstK<float> &Kf, const Pt &s) {
     const bool adj = M::gt(s.qc, K.qmin) || supersaturated<false>(K, Kf, s);
-    if (adj) return M::gt(K.T0, s.T) ? 1 : 2;
+    if (adj) return M::gt_any(K.T0, s.T) ? 1 : 2;
     bool act = M::gt(s.qr, K.qmin);
     if constexpr (!M::kWarm) {
       act = act || M::gt(s.qi, K.qmin) || M::gt(s.qs, K.qmin) || M::gt(s.qg, K.qmin);
-      act = act || (M::gt(K.Tnuc, s.T) && supersaturated<true>(K, Kf, s));
+      act = act || (M::gt_any(K.Tnuc, s.T) && supersaturated<true>(K, Kf, s));
     }
     return act ? 3 : 0;
   }
