@@ -1848,8 +1848,19 @@ __device__ __forceinline__ void stage_level(const KArgs &a, int k, int c, double
 // one addition per field and substep).
 // Measured (deep convection, 65 536 columns x 100 levels, dt = 10 s, mixed
 // step): 1.54 -> 0.95 ms.
+// More than pass_substeps substeps take further passes: the flux arrays lie in
+// local memory, and a kernel whose stack is above the 1024 bytes a thread that
+// the device has set aside makes it reserve more for every thread it can hold,
+// in steps of one substep too.  That is the FP64 form with sixth moments or
+// aerosol mass: 64 substeps a pass were 1568 bytes, 158 MB.
+// (Shorter arrays everywhere: 8 a pass, 65 536 x 100, dt = 10 s 853 -> 804 us,
+// but 20 000 x 60 219 -> 240, and at dt = 60 s 696 -> 825.)
 // prec: the species' surface mass; aprec: its aerosol mass (aerosol-mass
 // policies).  lvmask (may be null): bit k set for every level k it writes
+template <class M>
+__host__ __device__ constexpr int pass_substeps() {
+  return !M::kMixed && (M::kTri || M::kAero) ? 32 : 64;
+}
 template <class M, bool kTend>
 __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KParams &P, const LevelTab &lt, int c, int x,
                                                      int ns, double &prec, double &aprec, double *tend,
@@ -1869,99 +1880,102 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
   double *ap = state + (kTend ? 15 + x : 18 + x) * fs;   // aerosol mass in the species (aerosol-mass policies)
   const double dts = a.dt / ns;
   const float lim = 0.9999f * (float)ns;   // times dz / dt: below the speed limit in any rounding
-  R Fu[64], Gu[64];                        // kNsubMax substeps' fluxes out of the level above
-  R Xu[M::kTri || M::kAero ? 64 : 1];      // the sixth moment's or the aerosol mass's
-  for (int st = 0; st < ns; ++st) {
-    Fu[st] = Gu[st] = (R)0;
-    if (tri || aer) Xu[st] = (R)0;
-  }
-  bool inflow = false;   // some flux out of the level above
-  size_t o = (size_t)(a.nlev - 1) * a.pitch;
-  double qv = qp[o], nv = np[o], rv = __ldg(rhop + o), ev = tri ? zp[o] : aer ? ap[o] : 0.0;
-  for (int k = a.nlev - 1; k >= 0; --k) {
-    double q = qv, n = nv, e = ev;
-    const double rhod = rv;
-    const size_t ok = o;
-    if (k > 0) {   // the next level's values, in flight while this one is worked on
-      o -= a.pitch;
-      qv = qp[o];
-      nv = np[o];
-      rv = __ldg(rhop + o);
-      ev = tri ? zp[o] : aer ? ap[o] : 0.0;
+  constexpr int kPassSubsteps = pass_substeps<M>();
+  for (int s0 = 0; s0 < ns; s0 += kPassSubsteps) {
+    const int np1 = min(kPassSubsteps, ns - s0);        // this pass's substeps
+    R Fu[kPassSubsteps], Gu[kPassSubsteps];             // their fluxes out of the level above
+    R Xu[M::kTri || M::kAero ? kPassSubsteps : 1];      // the sixth moment's or the aerosol mass's
+    for (int st = 0; st < np1; ++st) {
+      Fu[st] = Gu[st] = (R)0;
+      if (tri || aer) Xu[st] = (R)0;
     }
-    if (!inflow && !(M::toR(q) > K.qmin)) continue;
-    const double dz = lt.dz[k];
-    const R rho = M::toR(rhod);
-    const R dfac = M::ex((R)0.4 * (K.lgrho0 - M::lg(rho)));
-    const R near = (R)lim * (R)lt.dzdt_f[k];
-    // a level's change by a flux divergence: the mixed form multiplies by
-    // dts / (rho dz); the FP64 form keeps dts dF / (rho dz), which gives back
-    // exactly what the speed limit lets out where it empties a level
-    const R sc = M::kMixed ? M::div(M::toRn(dts), M::toRn(rhod) * M::toRn(dz)) : (R)0;
-    auto change = [&](R dF) -> double {
-      if constexpr (M::kMixed) return M::toD(dF * sc);
-      else return M::div(dts * dF, rhod * dz);
-    };
-    bool wq = false, we = false;
-    inflow = false;
-    for (int st = 0; st < ns; ++st) {
-      const R qR = M::toR(q);
-      R F = 0, G = 0, X = 0;
-      if (qR > K.qmin) {
-        R vq, vn, vz = 0;
-        if (tri) {
-          Shape3<M>::fall_speeds(K, x, (R)1e30, qR, M::lg(qR), M::toR(n), M::toR(e), dfac, vq, vn, vz);
-        } else {
-          Ph::fall_speeds(K, (R)1e30, qR, M::toR(n), dfac, x, vq, vn);
-        }
-        if (!(M::mx(M::mx(vq, vn), vz) < near)) {
-          const R guard = M::toR(dz / dts);
-          vq = M::mn(vq, guard);
-          vn = M::mn(vn, guard);
-          vz = M::mn(vz, guard);
-        }
-        if constexpr (!M::kMixed) {
-          F = rhod * q * vq;
-          G = rhod * (n > 0.0 ? n : 0.0) * vn;
-          if (aer) X = rhod * e * vq;
-          if (tri) X = rhod * (e > 0.0 ? e : 0.0) * vz;
-        } else {
-          F = rho * qR * vq;
-          G = rho * M::mx(M::toR(n), (R)0) * vn;
-          if (aer) X = rho * M::toR(e) * vq;
-          if (tri) X = rho * M::mx(M::toR(e), (R)0) * vz;
-        }
+    bool inflow = false;   // some flux out of the level above
+    size_t o = (size_t)(a.nlev - 1) * a.pitch;
+    double qv = qp[o], nv = np[o], rv = __ldg(rhop + o), ev = tri ? zp[o] : aer ? ap[o] : 0.0;
+    for (int k = a.nlev - 1; k >= 0; --k) {
+      double q = qv, n = nv, e = ev;
+      const double rhod = rv;
+      const size_t ok = o;
+      if (k > 0) {   // the next level's values, in flight while this one is worked on
+        o -= a.pitch;
+        qv = qp[o];
+        nv = np[o];
+        rv = __ldg(rhop + o);
+        ev = tri ? zp[o] : aer ? ap[o] : 0.0;
       }
-      const R F1 = Fu[st], G1 = Gu[st];
-      if (tri || aer) {
-        const R X1 = Xu[st];
-        if (X != (R)0 || X1 != (R)0) {
-          e += change(X1 - X);
-          we = true;
-          eflag |= nonfinite(e);
+      if (!inflow && !(M::toR(q) > K.qmin)) continue;
+      const double dz = lt.dz[k];
+      const R rho = M::toR(rhod);
+      const R dfac = M::ex((R)0.4 * (K.lgrho0 - M::lg(rho)));
+      const R near = (R)lim * (R)lt.dzdt_f[k];
+      // a level's change by a flux divergence: the mixed form multiplies by
+      // dts / (rho dz); the FP64 form keeps the formula's order
+      const R sc = M::kMixed ? M::div(M::toRn(dts), M::toRn(rhod) * M::toRn(dz)) : (R)0;
+      auto change = [&](R dF) -> double {
+        if constexpr (M::kMixed) return M::toD(dF * sc);
+        else return M::div(dts * dF, rhod * dz);
+      };
+      bool wq = false, we = false;
+      inflow = false;
+      for (int st = 0; st < np1; ++st) {
+        const R qR = M::toR(q);
+        R F = 0, G = 0, X = 0;
+        if (qR > K.qmin) {
+          R vq, vn, vz = 0;
+          if (tri) {
+            Shape3<M>::fall_speeds(K, x, (R)1e30, qR, M::lg(qR), M::toR(n), M::toR(e), dfac, vq, vn, vz);
+          } else {
+            Ph::fall_speeds(K, (R)1e30, qR, M::toR(n), dfac, x, vq, vn);
+          }
+          if (!(M::mx(M::mx(vq, vn), vz) < near)) {
+            const R guard = M::toR(dz / dts);
+            vq = M::mn(vq, guard);
+            vn = M::mn(vn, guard);
+            vz = M::mn(vz, guard);
+          }
+          if constexpr (!M::kMixed) {
+            F = rhod * q * vq;
+            G = rhod * (n > 0.0 ? n : 0.0) * vn;
+            if (aer) X = rhod * e * vq;
+            if (tri) X = rhod * (e > 0.0 ? e : 0.0) * vz;
+          } else {
+            F = rho * qR * vq;
+            G = rho * M::mx(M::toR(n), (R)0) * vn;
+            if (aer) X = rho * M::toR(e) * vq;
+            if (tri) X = rho * M::mx(M::toR(e), (R)0) * vz;
+          }
         }
-        Xu[st] = X;
+        const R F1 = Fu[st], G1 = Gu[st];
+        if (tri || aer) {
+          const R X1 = Xu[st];
+          if (X != (R)0 || X1 != (R)0) {
+            e += change(X1 - X);
+            we = true;
+            eflag |= nonfinite(e);
+          }
+          Xu[st] = X;
+        }
+        if (F != (R)0 || F1 != (R)0 || G != (R)0 || G1 != (R)0) {
+          q += change(F1 - F);
+          n += change(G1 - G);
+          wq = true;
+          eflag |= nonfinite(q) | nonfinite(n);
+        }
+        Fu[st] = F;
+        Gu[st] = G;
+        inflow |= F != (R)0 || G != (R)0 || X != (R)0;
       }
-      if (F != (R)0 || F1 != (R)0 || G != (R)0 || G1 != (R)0) {
-        q += change(F1 - F);
-        n += change(G1 - G);
-        wq = true;
-        eflag |= nonfinite(q) | nonfinite(n);
+      if (wq) {
+        qp[ok] = q;
+        np[ok] = n;
+        if (lvmask) lvmask[k >> 5] |= 1u << (k & 31);
       }
-      Fu[st] = F;
-      Gu[st] = G;
-      inflow |= F != (R)0 || G != (R)0 || X != (R)0;
+      if (we) (tri ? zp : ap)[ok] = e;
     }
-    if (wq) {
-      qp[ok] = q;
-      np[ok] = n;
-      if (lvmask) lvmask[k >> 5] |= 1u << (k & 31);
+    for (int st = 0; st < np1; ++st) {
+      prec += M::toD(Fu[st]) * dts;
+      if (aer) aprec += M::toD(Xu[st]) * dts;
     }
-    if (we) (tri ? zp : ap)[ok] = e;
-  }
-  for (int st = 0; st < ns; ++st) {
-    prec += M::toD(Fu[st]) * dts;
-    if (aer) aprec += M::toD(Xu[st]) * dts;
   }
   return eflag;
 }
