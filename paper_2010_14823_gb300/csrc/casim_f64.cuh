@@ -23,9 +23,11 @@
 namespace casim_dev {
 
 constexpr int kF64Cols = 32;      // columns of a tile
-// levels of a chunk: as many as leave three blocks to an SM (8 fluxes a point
-// at 32 levels; 16 levels where points hand down 12).  Measured, cold step,
-// 8 / 16 / 24 / 32 levels: 6.46 / 6.18 / 6.07 / 6.04 ms
+// levels of a chunk.  At 32 levels of 8 fluxes a point the tile is 76 KB, two
+// blocks to an SM; at 16 levels of 12 fluxes (sixth moments, aerosol mass) three.
+// Measured, cold step, 24 levels (three blocks) / 32 levels: 65 536 x 100
+// stratus 5.84 / 5.96 ms, deep convection 10.97 / 10.47; 16 384 x 150 deep
+// convection 6.5 / 4.9 (an item of 150 levels is 7 chunks, or 5)
 template <class M>
 __host__ __device__ constexpr int f64_levels() {
   return M::kWarm || M::kTri || M::kAero ? 16 : 32;

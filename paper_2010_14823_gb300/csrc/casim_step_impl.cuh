@@ -12,7 +12,11 @@ namespace casim_dev {
 // 1: one thread per column).  A segment costs one extra level (its upper
 // neighbour, for the flux into it), so the column is split only as far as the
 // warps still fit in one resident wave, and into no more segments than it has
-// pairs of levels.  Measured, mixed cold step at 60 levels, 1 / 2 / 4 / 8 /
+// levels (256 columns of 32 levels, 16 / 32 segments: 23.4 / 20.7 us; of 16
+// levels, 8 / 16 segments: 23.7 / 20.4).  The wave is that of columns of a few
+// hundred levels: at 1024 levels three blocks fit, not kMinBlocks, but fewer
+// segments would be slower there (3 000 columns, 8 / 16 / 32 segments: 454 / 277 /
+// 273 us; 12 000: 944 / 868 / 870).  Measured, mixed cold step at 60 levels, 1 / 2 / 4 / 8 /
 // 16 / 32 segments: 20 000 columns 172 / 120 / 90 / 93 / 101 / 124 us, 5 000
 // columns - / 92 / 58 / 42 / 36 / 40 us; 256 columns x 50 levels 114 / 69 /
 // 40 / 28 / 22 / 16 us.  Beyond a wave splitting loses: 65 536 columns x 100
@@ -39,13 +43,22 @@ inline bool half_blocks(int warps, int nsm, int blocks_per_sm) {
   return 2 * ((half + nsm - 1) / nsm) < 4 * ((whole + nsm - 1) / nsm);   // warps of the fullest SM
 }
 
-// The FP64 sweep's segments per column group (1 to 8 blocks of a cluster): as
-// many as still fit in one resident wave, at least 4 levels each.
-inline int f64_segments(unsigned groups, int nlev, int nsm, int blocks_per_sm) {
-  const unsigned room = (unsigned)(nsm * blocks_per_sm);
-  int n = 1;
-  while (n < 8 && 8 * n <= nlev && 2 * n * groups <= room) n *= 2;
-  return n;
+// The FP64 sweep's segments per column group (1, 2, 4 or 8 blocks of a
+// cluster, at least 4 levels each).  Four or eight, if that gives at most
+// split_blocks blocks per SM (cold step: 1.5 resident waves); two, if they are
+// resident at once, since twice two half columns take longer than one wave of
+// whole ones.  Measured, cold step, us with 1 / 2 / 4 / 8 segments:
+//   columns x levels   deep convection x 60        stratus x 150
+//   1 824              577 / 404 / 378 / 327       938 /  589 /  575 /  475
+//   2 400              537 / 370 / 382 / 394      1044 /  593 /  638 /  539
+//   3 648              545 / 608 / 626 / 518      1044 /  902 /  964 /  732
+//   4 864              546 / 609 / 696 / 662      1050 /  908 / 1132 /  908
+//   6 400              856 /1065 / 855 / 814      1454 / 1693 / 1434 / 1164
+//   9 600              888 /1171 /1168 /1153      1467 / 1758 / 1945 / 1635
+inline int f64_segments(unsigned groups, int nlev, int nsm, int resident, int split_blocks) {
+  for (int n = 8; n > 2; n /= 2)
+    if (4 * n <= nlev && n * groups <= (unsigned)(nsm * split_blocks)) return n;
+  return 8 <= nlev && 2 * groups <= (unsigned)(nsm * resident) ? 2 : 1;
 }
 
 // grid.x column groups; the levels of a column shared by clusters of grid.y blocks
@@ -93,6 +106,9 @@ cudaError_t StepKernels<PMix, PF64>::allow_smem() {
 
 template <class PMix, class PF64>
 cudaError_t StepKernels<PMix, PF64>::launch(const StepLaunch &l, const KArgs &args, const KParams &kp) {
+  // the kernels' blocks per SM fit its shared memory (228 KB, 1 KB of each block reserved)
+  static_assert(PF64::kMinBlocks * (f64_smem_bytes<PF64>(150) + 1024) <= 228 * 1024, "FP64 blocks per SM");
+  static_assert(PMix::kMinBlocks * (step_smem_bytes<PMix>(150) + 1024) <= 228 * 1024, "mixed blocks per SM");
   KArgs a = args;
   const bool line = l.line && l.mixed;
   const unsigned groups = (unsigned)((a.ncols + kF64Cols - 1) / kF64Cols);   // FP64 blocks
@@ -107,7 +123,7 @@ cudaError_t StepKernels<PMix, PF64>::launch(const StepLaunch &l, const KArgs &ar
   }
   if (!l.mixed) {
     // FP64: blocks of 32 columns, a cluster of segments where they are few
-    const dim3 grid(groups, (unsigned)f64_segments(groups, a.nlev, l.nsm, PF64::kMinBlocks));
+    const dim3 grid(groups, (unsigned)f64_segments(groups, a.nlev, l.nsm, PF64::kMinBlocks, PF64::kSplitBlocks));
     const size_t smem = f64_smem_bytes<PF64>(a.nlev);
     return l.tend ? step_launch(k_step<PF64, true>, grid, smem, l.stream, a, kp, l.tend)
                   : step_launch(k_step<PF64, false>, grid, smem, l.stream, a, kp, nullptr);
