@@ -751,17 +751,21 @@ struct F64T {
   using P = Phys<M>;
 
   // q > q_s(T, p) over liquid (ice: over ice).  Decided in FP32 where the two
-  // differ by more than 1e-4 of q_s (the FP32 value is good to ~2e-6), else by
-  // the FP64 expression.
+  // differ by more than 1e-4 of q_s, else by the FP64 expression.  The FP32 q_s
+  // is good to 1.0e-5 (at 128 K; T rounded to FP32 moves it by 6e-6 there) for
+  // temperatures of 128 to 512 K and a vapour pressure that takes up at most
+  // half of p in p - (1 - eps) es; outside, FP64 decides.
   template <bool kIce>
   static __device__ __forceinline__ bool supersaturated(const ConstK<double> &K, const ConstK<float> &Kf, const Pt &s) {
-    if (max(max(hiabs(s.T), hiabs(s.p)), hiabs(s.qv)) < kF32RangeHi) {
+    const bool t_ok = (unsigned)__double2hiint(s.T) - 0x40600000u < 0x00200000u;   // 128 <= T < 512
+    if (t_ok && max(hiabs(s.p), hiabs(s.qv)) < kF32RangeHi) {
       const float T = d2f(s.T), p = d2f(s.p), q = d2f(s.qv);
       const float tc = T - Kf.T0;
       const float es = kIce ? Kf.esi0 * PolicyMix::exp(__fdividef(Kf.esia * (T - Kf.esit), T - Kf.esib))
                             : Kf.esl0 * PolicyMix::exp(__fdividef(Kf.esla * tc, tc + Kf.eslb));
-      const float qs = __fdividef(Kf.eps * es, p - Kf.ome * es);
-      if (qs > 0.f) {
+      const float den = p - Kf.ome * es;
+      const float qs = __fdividef(Kf.eps * es, den);
+      if (den > 0.5f * p && qs > 0.f) {
         if (q > 1.0001f * qs) return true;
         if (q < 0.9999f * qs) return false;
       }
