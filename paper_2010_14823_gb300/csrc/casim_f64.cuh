@@ -313,24 +313,35 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
       }
     }
   } else {
-    // the segments' Courant numbers meet; the species are dealt to the
-    // segments and warps (with aerosol mass one thread takes them all: their
-    // surface fluxes of aerosol add up in order)
-    if (sg.nseg > 1) {
-      split_arrive();
-      split_wait();
-    }
-    const int c = t.col[lane];
-    for (int x = 0; x < kSed; ++x) {
-      const bool mine = M::kAero ? sg.seg == 0 && warp == 0 : x % sg.nseg == sg.seg && warp == x % (B >> 5);
-      if (!mine || c < 0) continue;
-      double cmax = 0.0;
-      for (int j = 0; j < sg.nseg; ++j) {
-        const double v = sg.nseg > 1 ? sg.slot(reinterpret_cast<const double *>(&t.cmax[x][lane]), j)
-                                     : __longlong_as_double((long long)t.cmax[x][lane]);
-        cmax = v > cmax ? v : cmax;
+    // the segments' Courant numbers meet in the top segment's block, whose warps
+    // take a species each (with aerosol mass one thread takes them all: their
+    // surface fluxes of aerosol add up in order).  The other blocks leave, so that
+    // a cluster of a later wave need not wait for the sweeps (1 824 columns x 60,
+    // dt = 10 s, 8 segments: 2.80 -> 1.68 ms, source terms 2.83 -> 1.80).
+    auto barrier = [&] {
+      if (sg.nseg > 1) {
+        split_arrive();
+        split_wait();
       }
-      int ns = (int)ceil(cmax / P.c_max);
+    };
+    barrier();
+    const int c = t.col[lane];
+    double cmax[4] = {0.0, 0.0, 0.0, 0.0};
+    if (sg.seg == 0) {
+#pragma unroll
+      for (int x = 0; x < kSed; ++x) {
+        for (int j = 0; j < sg.nseg; ++j) {
+          const double v = sg.nseg > 1 ? sg.slot(reinterpret_cast<const double *>(&t.cmax[x][lane]), j)
+                                       : __longlong_as_double((long long)t.cmax[x][lane]);
+          cmax[x] = v > cmax[x] ? v : cmax[x];
+        }
+      }
+    }
+    barrier();   // the slots have been read
+    for (int x = 0; x < kSed; ++x) {
+      const bool mine = sg.seg == 0 && warp == (M::kAero ? 0 : x % (B >> 5));
+      if (!mine || c < 0) continue;
+      int ns = (int)ceil((x == 0 ? cmax[0] : x == 1 ? cmax[1] : x == 2 ? cmax[2] : cmax[3]) / P.c_max);
       if (ns < 1) ns = 1;
       if (ns > 64) { ns = 64; eflag |= 2u; }
       double pr = 0.0;
@@ -347,14 +358,10 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
       for (int j = 0; j < kSed; ++j)
         if (x == j) prec[j] = pr;
     }
-    if (sg.nseg > 1) {   // the slots have been read and the sweeps' results stored
-      split_arrive();
-      split_wait();
-    }
     __syncthreads();
     if constexpr (kTend) {
-      for (int i = tid; i < (sg.ktop() - sg.kbot() + 1) * kF64Cols; i += B) {
-        const int k = sg.ktop() - (i >> 5);
+      for (int i = tid; i < (sg.seg == 0 ? a.nlev * kF64Cols : 0); i += B) {
+        const int k = i >> 5;
         if (c < 0) continue;
         const size_t o = (size_t)k * a.pitch + c;
 #pragma unroll
