@@ -261,6 +261,7 @@ struct PolicyMix {
   static constexpr bool kAero = false;
   static constexpr bool kTri = false;
   static constexpr int kMinBlocks = 5;   // measured: 4 / 5 / 6 -> 2.07 / 1.94 / 1.99 ms per 512x512x150 step
+  static constexpr int kSplitBlocks = 5;   // step_segments
   static __device__ __forceinline__ const ConstK<float> &K(const KParams &p) { return p.f; }
   static __device__ __forceinline__ R toR(double x) { return d2f(x); }
   static __device__ __forceinline__ R toRn(double x) { return d2f_rn(x); }
@@ -1415,6 +1416,7 @@ struct PolicyMixWarm : PolicyMix {
   // measured on 512x512x150 stratus: 6 / 7 / 8 -> 1.062 / 0.961 / 0.940 ms per step
   // (64 registers, no spills at 8); the triple-moment warm form: 1.495 / 1.416 / 1.385
   static constexpr int kMinBlocks = 8;
+  static constexpr int kSplitBlocks = 8;
 };
 // The warm configuration with activated-aerosol mass (Section 2: aerosol
 // carried in the cloud once activated and returned when the water
@@ -1429,6 +1431,7 @@ struct PolicyMixWarmAero : PolicyMixWarm {
   static constexpr bool kAero = true;
   // measured: 6 / 7 / 8 -> 1.358 / 1.235 / 1.263 ms per step (36 B spilled at 8)
   static constexpr int kMinBlocks = 7;
+  static constexpr int kSplitBlocks = 5;
 };
 // The warm configuration with triple-moment rain (Section 2: CASIM is a
 // three-moment scheme): field 16 of the state is the rain's sixth moment z
@@ -1440,6 +1443,7 @@ struct PolicyF64Warm3 : PolicyF64Warm {
 };
 struct PolicyMixWarm3 : PolicyMixWarm {
   static constexpr bool kTri = true;
+  static constexpr int kSplitBlocks = 5;
 };
 // The cold configuration with triple-moment r, i, s, g: fields 16..19 are
 // their sixth moments.
@@ -1456,10 +1460,12 @@ struct PolicyF64Aero : PolicyF64 {
 struct PolicyMixAero : PolicyMix {
   static constexpr bool kAero = true;
   static constexpr int kMinBlocks = 4;   // measured: 4 / 5 -> 3.41 / 3.88 ms per stratus step
+  static constexpr int kSplitBlocks = 4;
 };
 struct PolicyMix3 : PolicyMix {
   static constexpr bool kTri = true;
   static constexpr int kMinBlocks = 4;   // measured: 4 / 5 -> 4.69 / 5.50 ms per stratus step
+  static constexpr int kSplitBlocks = 4;
 };
 
 // ---------------------------------------------------------------- kernels
@@ -1860,20 +1866,23 @@ __device__ __forceinline__ void stage_level(const KArgs &a, int k, int c, double
 // one addition per field and substep).
 // Measured (deep convection, 65 536 columns x 100 levels, dt = 10 s, mixed
 // step): 1.54 -> 0.95 ms.
-// More than pass_substeps substeps take further passes: the flux arrays lie in
+// More than kPassSubsteps substeps take further passes: the flux arrays lie in
 // local memory, and a kernel whose stack is above the 1024 bytes a thread that
 // the device has set aside makes it reserve more for every thread it can hold,
 // in steps of one substep too.  That is the FP64 form with sixth moments or
 // aerosol mass: 64 substeps a pass were 1568 bytes, 158 MB.
 // (Shorter arrays everywhere: 8 a pass, 65 536 x 100, dt = 10 s 853 -> 804 us,
 // but 20 000 x 60 219 -> 240, and at dt = 60 s 696 -> 825.)
+// (the mixed warm triple-moment form takes 16 with one thread per column:
+// 262 144 x 60, dt = 10 s 2.09 -> 1.53 ms)
+template <class M, bool kSplit>
+__host__ __device__ constexpr int pass_substeps() {
+  if (!M::kMixed) return M::kTri || M::kAero ? 32 : 64;
+  return M::kWarm && M::kTri && !kSplit ? 16 : 64;
+}
 // prec: the species' surface mass; aprec: its aerosol mass (aerosol-mass
 // policies).  lvmask (may be null): bit k set for every level k it writes
-template <class M>
-__host__ __device__ constexpr int pass_substeps() {
-  return !M::kMixed && (M::kTri || M::kAero) ? 32 : 64;
-}
-template <class M, bool kTend>
+template <class M, bool kTend, int kPassSubsteps>
 __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KParams &P, const LevelTab &lt, int c, int x,
                                                      int ns, double &prec, double &aprec, double *tend,
                                                      unsigned *lvmask) {
@@ -1892,7 +1901,6 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
   double *ap = state + (kTend ? 15 + x : 18 + x) * fs;   // aerosol mass in the species (aerosol-mass policies)
   const double dts = a.dt / ns;
   const float lim = 0.9999f * (float)ns;   // times dz / dt: below the speed limit in any rounding
-  constexpr int kPassSubsteps = pass_substeps<M>();
   for (int s0 = 0; s0 < ns; s0 += kPassSubsteps) {
     const int np1 = min(kPassSubsteps, ns - s0);        // this pass's substeps
     R Fu[kPassSubsteps], Gu[kPassSubsteps];             // their fluxes out of the level above
@@ -2283,7 +2291,8 @@ __device__ __forceinline__ unsigned sweep_column(const KArgs &a, const KParams &
       if (ns > 64) { ns = 64; eflag |= 2u; }
       if constexpr (kStats) cs->nsub[x] = ns;
       double pr = 0.0;
-      eflag |= sediment_species<M, kTend>(a, P, lt, c, x, ns, pr, prec[4], tend, kStats ? lvmask : nullptr);
+      eflag |= sediment_species<M, kTend, pass_substeps<M, kSplit>()>(a, P, lt, c, x, ns, pr, prec[4], tend,
+                                                                       kStats ? lvmask : nullptr);
 #pragma unroll
       for (int i = 0; i < kSed; ++i)
         if (x == i) prec[i] = pr;

@@ -338,6 +338,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
       }
     }
     barrier();   // the slots have been read
+    constexpr int kPass = pass_substeps<M, false>();
     for (int x = 0; x < kSed; ++x) {
       const bool mine = sg.seg == 0 && warp == (M::kAero ? 0 : x % (B >> 5));
       if (!mine || c < 0) continue;
@@ -348,11 +349,11 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
       if constexpr (kStats) {
         unsigned lv[(kMaxLev + 31) / 32] = {};
         st->nsub[x][lane] = ns;
-        eflag |= sediment_species<M, kTend>(a, P, lt, c, x, ns, pr, prec[4], tend, lv);
+        eflag |= sediment_species<M, kTend, kPass>(a, P, lt, c, x, ns, pr, prec[4], tend, lv);
         for (int w = 0; w < (kMaxLev + 31) / 32; ++w)
           if (lv[w]) atomicOr(&st->lv[lane][w], lv[w]);
       } else {
-        eflag |= sediment_species<M, kTend>(a, P, lt, c, x, ns, pr, prec[4], tend, nullptr);
+        eflag |= sediment_species<M, kTend, kPass>(a, P, lt, c, x, ns, pr, prec[4], tend, nullptr);
       }
 #pragma unroll
       for (int j = 0; j < kSed; ++j)

@@ -21,6 +21,11 @@ namespace casim_dev {
 // columns - / 92 / 58 / 42 / 36 / 40 us; 256 columns x 50 levels 114 / 69 /
 // 40 / 28 / 22 / 16 us.  Beyond a wave splitting loses: 65 536 columns x 100
 // triple-moment 837 / 985 / 937 us, 262 144 x 150 cold 1927 / 2022 / 2060 us.
+// The warm forms with a third field stop at five blocks per SM, not at the wave's
+// seven and eight: in steps of several substeps their full SMs leave the flux
+// arrays too little cache (65 536 x 60, 1 / 2 segments, aerosol mass: dt = 1 s
+// 199 / 187 us, dt = 10 s 385 / 660; sixth moments, 100 levels, dt = 10 s: 937 /
+// 1223).
 // A state in host memory saturates the host link with fewer warps
 // (20 000 x 60: 834 / 840 / 853 us).
 inline int step_segments(int ncols, int nlev, int nsm, int blocks_per_sm, bool line) {
@@ -128,7 +133,7 @@ cudaError_t StepKernels<PMix, PF64>::launch(const StepLaunch &l, const KArgs &ar
     return l.tend ? step_launch(k_step<PF64, true>, grid, smem, l.stream, a, kp, l.tend)
                   : step_launch(k_step<PF64, false>, grid, smem, l.stream, a, kp, nullptr);
   }
-  const int n = step_segments(a.ncols, a.nlev, l.nsm, PMix::kMinBlocks, line);
+  const int n = step_segments(a.ncols, a.nlev, l.nsm, PMix::kSplitBlocks, line);
   const size_t smem = step_smem_bytes<PMix>(a.nlev);
   const bool half = n == 1 && !line && half_blocks((a.ncols + 31) / 32, l.nsm, PMix::kMinBlocks);
   auto go = [&](auto *one, auto *split, auto *small) {
