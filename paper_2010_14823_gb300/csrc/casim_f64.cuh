@@ -338,7 +338,7 @@ __device__ __forceinline__ unsigned f64_sweep(const KArgs &a, const KParams &P, 
       }
     }
     barrier();   // the slots have been read
-    constexpr int kPass = pass_substeps<M, false>();
+    constexpr int kPass = kStats ? 32 : pass_substeps<M, false>();   // (the statistics hold local memory too)
     for (int x = 0; x < kSed; ++x) {
       const bool mine = sg.seg == 0 && warp == (M::kAero ? 0 : x % (B >> 5));
       if (!mine || c < 0) continue;

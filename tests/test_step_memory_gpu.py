@@ -33,7 +33,7 @@ casim.casim_free(ctx)
 
 
 @pytest.mark.parametrize("precision", ["CASIM_FP64", "CASIM_MIXED"])
-@pytest.mark.parametrize("names,nf", [((), 16), (("CASIM_AEROSOL",), 22), (("CASIM_THREE_MOMENT",), 20)])
+@pytest.mark.parametrize("names,nf", [((), 16), (("CASIM_STATS",), 16), (("CASIM_AEROSOL",), 22), (("CASIM_THREE_MOMENT",), 20)])
 def test_first_step_takes_no_memory(precision, names, nf):
     from paper_2010_14823_gb300 import casim
     flags = sum(getattr(casim, n) for n in names)
