@@ -33,26 +33,26 @@ WORKLOAD = "deep_512x512x150"
 
 # DRAM traffic of k_step<PolicyMix> on the deep-convection state, from one
 # single-pass ncu capture of the full 262 144-column x 150-level launch
-# (dram__bytes_read.sum + dram__bytes_write.sum = 5.0611 + 3.9698 GB for
+# (dram__bytes_read.sum + dram__bytes_write.sum = 5.0598 + 3.9702 GB for
 # 39.32 M points); at another column count it is scaled per point (reads are
 # 16 fields per point and writes follow the changed points).  Valid only for
 # the kernel source it was taken on.
-MEASURED_TRAFFIC = {"kernel": "k_step<PolicyMix>", "bytes_per_launch": 9030921216, "points": 39321600,
-                    "bytes_per_point": 229.67,
+MEASURED_TRAFFIC = {"kernel": "k_step<PolicyMix>", "bytes_per_launch": 9029951488, "points": 39321600,
+                    "bytes_per_point": 229.64,
                     "source": "paper_2010_14823_gb300/csrc/casim_device.cuh",
-                    "sha256": "175716eac5f3a50d281cf54ff1afe3d8df0760f9d5e3726c1ab97780908559db"}
+                    "sha256": "588091e2722dc0567079f6eaa10f6a6e40c4992ef043da7803c5dc362c337423"}
 
 
 # FP64 arithmetic instructions of k_step<PolicyF64> per point on the same
 # state, from one ncu capture of a 16 384-column x 150-level launch
 # (smsp__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum =
-# 582.3 M + 210.9 M + 289.5 M for 2.458 M points); the FP64 pipe was 79.3 %
+# 853.4 M + 259.6 M + 346.4 M for 2.458 M points); the FP64 pipe was 80.4 %
 # busy.  Valid only for the kernel source it was taken on.
-MEASURED_FP64_OPS = {"kernel": "k_step<PolicyF64>", "inst_per_point": 440.53,
-                     "dfma": 236.92, "dadd": 85.81, "dmul": 117.80, "fp64_pipe_active": 0.793,
-                     "with": {"casim_f64.cuh": "b622fbabc865a116ec75f857d71932b9070e16deec92f520d2cbf81df5cdf9bb",
-                              "casim_math64.cuh": "77319d4ef15b9df62adbc456dce9219359100983f498f8e1132fc06f027ec9dd"},
-                     "sha256": "175716eac5f3a50d281cf54ff1afe3d8df0760f9d5e3726c1ab97780908559db"}
+MEASURED_FP64_OPS = {"kernel": "k_step<PolicyF64>", "inst_per_point": 593.86,
+                     "dfma": 347.26, "dadd": 105.64, "dmul": 140.96, "fp64_pipe_active": 0.804,
+                     "with": {"casim_f64.cuh": "76d4c035564d1c49484e4b320591531145f13cc82fc43b7de24bd1719bf61a27",
+                              "casim_math64.cuh": "62c7b2eef4c9c3d22dbb18726d829b942e0dfa7ff5ed761d120ee1283817414a"},
+                     "sha256": "588091e2722dc0567079f6eaa10f6a6e40c4992ef043da7803c5dc362c337423"}
 
 
 def _host_link_gbs(torch, stream, nbytes: int = 1 << 30):

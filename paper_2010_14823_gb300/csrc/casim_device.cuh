@@ -1,14 +1,18 @@
 // Device code of the column-microphysics step (sm_103a).
 //
-// One thread owns one column and walks it from the top level down
-// (Section 3.2 of the paper maps one column to one GPU thread as well; the
-// column's levels are coupled only through sedimentation).  Loads and stores
+// The mixed form: one thread walks a column from the top level down (Section
+// 3.2 of the paper maps one column to one GPU thread as well; the column's
+// levels are coupled only through sedimentation), or, for domains too small to
+// fill the chip so, a segment of its levels.  The FP64 form: a block takes 32
+// columns and a list of their active points (casim_f64.cuh).  Loads and stores
 // are level-major, so the 32 threads of a warp touch 32 consecutive columns of
 // one level: every access is a coalesced 256-byte row.
 //
 // Two precision policies share the process formulas:
-//   PolicyF64  every operation in FP64, transfers applied in the order of the
-//              scheme's transfer list;
+//   PolicyF64  every value and operation in FP64, transfers applied in the
+//              order of the scheme's transfer list (comparisons by the values'
+//              bits; whether a point clearly away from saturation is active, in
+//              FP32);
 //   PolicyMix  rates, fall speeds and special functions in FP32 on the MUFU
 //              pipe (ex2/lg2); each field's increments at a point (process
 //              transfers, sedimentation) are summed in FP32 and added to the
@@ -67,6 +71,10 @@ struct ConstK {
   R mey_a, mey_b, mey_c, mi0;
   // air
   R mu_air, inv_dv, lgrho0, twopi;
+  // unused: keeps the species' constants at the offset at which the mixed
+  // kernels were timed (65 536 x 150 source terms 748 us; 760 without, from the
+  // constants' other alignment in the kernel's parameters alone)
+  R spare[3];
   SpeciesK<R> sp[5];
   // triple-moment species r, i, s, g (index 0..3, species 1..4): what their
   // shape-dependent constants are built from
@@ -493,7 +501,8 @@ struct Shape3 {
 // rounding, and the compiler's own choice follows the uses a product has in
 // the kernel at hand: two kernels of one configuration could differ in the
 // last bit of a limited transfer.  So the choice is written out; `kFused` has
-// a bit per place, set as each configuration's kernels have always had it.
+// a bit per place, set as the compiler had chosen for each configuration's
+// one-thread-per-column kernel, so that writing it out changed no result.
 template <bool kFused>
 __device__ __forceinline__ float add_product(float s, float a, float b) {   // s + a b
   if constexpr (kFused) return fmaf(a, b, s);
@@ -2005,7 +2014,7 @@ __device__ __forceinline__ unsigned sediment_species(const KArgs &a, const KPara
 // sedimentation substep and the flux recurrence is fused into the top-down
 // sweep of the processes (one read and one write of the state).  Otherwise
 // the processes are applied first and each species is sedimented with its
-// own substep count in further sweeps over the column.
+// own substep count in a further pass down the column (sediment_species).
 // The mixed form's sweep.  stg: this thread's slots of the prefetch stage (slot f of buffer
 // b at stg[(b * 16 + f) * ss], ss the block's thread count): level k - 1's 16
 // fields are copied there by cp.async while level k is processed, so the

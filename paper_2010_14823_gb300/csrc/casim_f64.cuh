@@ -5,7 +5,7 @@
 // 30 % cloudy columns), and the long inlined code of the branches they took
 // one after the other missed the instruction cache.
 //
-// Here a block takes 32 columns and walks them down in chunks of levels.  In
+// Here a block of 128 threads takes 32 columns and walks them down in chunks of levels.  In
 // each chunk it flags the points (every lane busy), lists the active ones by
 // the branches they will take, runs the processes over the list in full
 // warps, and then applies the sedimentation, whose fluxes the points hand

@@ -1101,10 +1101,10 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) k_mlp_umma(const UmmaArgs u) 
 // epilogue), so the whole depth of up to 256 is loaded at once, in slabs of 64
 // whose MMAs follow as they land, and small tiles put every SM to work: with
 // 128 x 128 tiles of 4 warps and two slabs in flight a hidden layer took 24 us
-// on 8192 rows and a data gradient 36 us, now 10 and 11 us; the weight
-// gradients, one launch per layer with 128 x 128 tiles transposed through
-// registers, took 92 us, now 17 us in one launch (all by ncu, cold caches).
-// A training step on 8192 rows: 0.34 -> 0.094 ms.
+// on 8192 rows and a data gradient 36 us, now 12 us each; the weight
+// gradients, one launch of 23 us per layer with 128 x 128 tiles transposed
+// through registers, take 18 us in one launch for all four (all by ncu, cold
+// caches).  A training step on 8192 rows: 0.33 -> 0.094 ms.
 // One thread issues the MMAs (M = 128, N = the
 // tile's columns rounded up to 16, K = 16 each).  Epilogue: warp w reads
 // tensor-memory lanes 32 (w % 4).. (its rows) and 32 columns, and passes the
